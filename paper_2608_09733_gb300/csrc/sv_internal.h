@@ -182,6 +182,11 @@ template <typename R>
 cudaError_t launch_expect_terms(const Cx<R>* state, int n, const sv_pauli_term* terms, int n_terms, double* scratch,
                                 size_t scratch_doubles, double* out, cudaStream_t stream);
 size_t expect_z_all_scratch_doubles(int n);
+// The same for `batch` states back to back: out holds batch x (n + 1) doubles.
+template <typename R>
+cudaError_t launch_expect_z_batch(const Cx<R>* states, int n, int batch, double* scratch, size_t scratch_doubles,
+                                  double* out, cudaStream_t stream);
+size_t expect_z_batch_scratch_doubles(int n, int batch, size_t amp_bytes);
 
 size_t expect_terms_scratch_doubles(int n, int n_terms);
 

@@ -21,9 +21,14 @@
 // reductions.  (Warp sums in double took most of the kernel's time: the FP64
 // pipe of this part runs a warp-wide add in about 16 cycles.)  complex128
 // accumulates in double throughout.
-// The grid writes one partial per block and a one-block kernel adds them in a
+// The grid writes one partial per block and a second kernel adds them in a
 // fixed order, so results are identical run to run.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <map>
+#include <utility>
+#include <vector>
 
 #include "sv_internal.h"
 
@@ -35,6 +40,7 @@ constexpr int kRedThreads = 256;
 constexpr int kRedWarps = kRedThreads / 32;
 constexpr int kJ = 32;          // vectors per lane per chunk
 constexpr int kMaxTermsPerPass = 16;
+constexpr int kMaxTermSlots = 128;  // terms whose partials one finish launch adds up
 
 int red_grid() { return device_sm_count() * 4; }
 
@@ -54,13 +60,35 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ float warp_sum(float v) {
+
+// Sums of W values over the warp's lanes: each step hands half of the values
+// to the partner lane, so W sums take W + log2(32 / W) - 1 adds a lane instead
+// of 5 W (an FP64 add occupies the SM's FP64 pipe for about 16 cycles).  The
+// lane ends with the sum of value lane / (32 / W), added as the tree that
+// warp_sum adds.
+template <int W, int O = 16, typename T>
+__device__ __forceinline__ T warp_fold(T (&a)[W], int lane) {
+  if constexpr (W == 1) {
+    T v = a[0];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+    for (int o = O; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  } else {
+    T b[W / 2];
+    const bool hi = lane & O;
+#pragma unroll
+    for (int k = 0; k < W / 2; k++) {
+      const T keep = hi ? a[k + W / 2] : a[k], send = hi ? a[k] : a[k + W / 2];
+      b[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+    return warp_fold<W / 2, O / 2>(b, lane);
+  }
 }
 
 // ------------------------------------------------------------ <Z_q> for all q
+//
+// grid.y is the state of a batch (one for a single read-out): state b starts
+// at state + (b << n), its partial rows at (b * gridDim.x) rows.
 
 // A = amplitudes per 16-byte vector (2 for complex64, 1 for complex128).
 // Chunk = 32 lanes x kJ vectors x A amplitudes; chunk bits C = log2(1024 A).
@@ -72,62 +100,67 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_z_all(const Cx<R>* __res
   constexpr int C = EB + 5 + 5;         // chunk bits
   using T = typename Acc<R>::T;
   __shared__ double red[kRedWarps][SV_MAX_QUBITS + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, block_warps = blockDim.x >> 5;
   const uint64_t nchunks = 1ull << (n - C);
-  const uint64_t gwarp = (uint64_t)blockIdx.x * kRedWarps + warp;
-  const uint64_t nwarps = (uint64_t)gridDim.x * kRedWarps;
+  const uint64_t gwarp = (uint64_t)blockIdx.x * block_warps + warp;
+  const uint64_t nwarps = (uint64_t)gridDim.x * block_warps;
+  state += (uint64_t)blockIdx.y << n;
   double accq0 = 0.0, accq1 = 0.0, acct = 0.0;  // qubits lane and lane + 32; total
   for (uint64_t ch = gwarp; ch < nchunks; ch += nwarps) {
     const uint4* src = reinterpret_cast<const uint4*>(state + (ch << C));
-    T tot = 0, e1 = 0, jb0 = 0, jb1 = 0, jb2 = 0, jb3 = 0, jb4 = 0;
+    // the lane's sums: total, element 1, iteration bits 0..4 set, lane bits
+    // 0..4 set (the total where the bit is set)
+    T v[16];
 #pragma unroll
-    for (int j = 0; j < kJ; j++) {
-      uint4 w = __ldg(src + j * 32 + lane);
-      T p;
-      if constexpr (A == 2) {
+    for (int k = 0; k < 16; k++) v[k] = 0;
+    if constexpr (A == 2) {
+#pragma unroll
+      for (int j = 0; j < kJ; j++) {
+        uint4 w = __ldg(src + j * 32 + lane);
         float2 a = *reinterpret_cast<float2*>(&w.x), b = *reinterpret_cast<float2*>(&w.z);
         T p0 = fmaf(a.x, a.x, a.y * a.y), p1 = fmaf(b.x, b.x, b.y * b.y);
-        e1 += p1;
-        p = p0 + p1;
-      } else {
+        v[1] += p1;
+        const T p = p0 + p1;
+        v[0] += p;
+#pragma unroll
+        for (int b2 = 0; b2 < 5; b2++)
+          if ((j >> b2) & 1) v[2 + b2] += p;
+      }
+    } else {
+      // pairwise over the iteration bits: 62 adds for the total and the five
+      // bit sums of 32 values, against 112 added one by one (FP64 pipe bound)
+      T p[kJ];
+#pragma unroll
+      for (int j = 0; j < kJ; j++) {
+        uint4 w = __ldg(src + j * 32 + lane);
         double2 a = *reinterpret_cast<double2*>(&w);
-        p = fma(a.x, a.x, a.y * a.y);
+        p[j] = fma(a.x, a.x, a.y * a.y);
       }
-      tot += p;
-      if (j & 1) jb0 += p;
-      if (j & 2) jb1 += p;
-      if (j & 4) jb2 += p;
-      if (j & 8) jb3 += p;
-      if (j & 16) jb4 += p;
-    }
-    // reduce the lanes' runs across the warp (in the run's precision), then
-    // into double
-    const double t = (double)warp_sum(tot);
-    const double v_e1 = EB ? (double)warp_sum(e1) : 0.0;
-    const double v_j[5] = {(double)warp_sum(jb0), (double)warp_sum(jb1), (double)warp_sum(jb2),
-                           (double)warp_sum(jb3), (double)warp_sum(jb4)};
-    double v_l[5];
 #pragma unroll
-    for (int b = 0; b < 5; b++) v_l[b] = (double)warp_sum(((lane >> b) & 1) ? tot : T(0));
-    // lane q picks S_q for its qubits q = lane and lane + 32
+      for (int b2 = 0; b2 < 5; b2++) {
 #pragma unroll
-    for (int rep = 0; rep < 2; rep++) {
-      const int q = lane + 32 * rep;
-      if (q >= n) continue;
-      double sq;
-      if (q >= C) {
-        sq = ((ch >> (q - C)) & 1ull) ? t : 0.0;
-      } else if (EB && q == 0) {
-        sq = v_e1;
-      } else if (q < EB + 5) {
-        int b = q - EB;
-        sq = b == 0 ? v_l[0] : b == 1 ? v_l[1] : b == 2 ? v_l[2] : b == 3 ? v_l[3] : v_l[4];
-      } else {
-        int b = q - EB - 5;
-        sq = b == 0 ? v_j[0] : b == 1 ? v_j[1] : b == 2 ? v_j[2] : b == 3 ? v_j[3] : v_j[4];
+        for (int j = 0; j < (kJ >> (b2 + 1)); j++) {
+          v[2 + b2] += p[2 * j + 1];
+          p[j] = p[2 * j] + p[2 * j + 1];
+        }
       }
-      if (rep == 0) accq0 += sq; else accq1 += sq;
+      v[0] = p[0];
     }
+#pragma unroll
+    for (int b = 0; b < 5; b++) v[7 + b] = ((lane >> b) & 1) ? v[0] : T(0);
+    // the sum of value k sits in lanes 2 k and 2 k + 1 (in the run's
+    // precision), then into double
+    const double sum = (double)warp_fold(v, lane);
+    const double t = __shfl_sync(0xffffffffu, sum, 0);
+    // lane q picks S_q for its qubits q = lane and lane + 32: bits inside the
+    // chunk from the lane holding their sum, bits above it from the chunk index
+    const int k = (EB && lane == 0) ? 1 : lane < EB + 5 ? 7 + lane - EB : 2 + lane - EB - 5;
+    const double in_chunk = __shfl_sync(0xffffffffu, sum, lane < C ? 2 * k : 0);
+    if (lane < C)
+      accq0 += in_chunk;
+    else if (lane < n)
+      accq0 += ((ch >> (lane - C)) & 1ull) ? t : 0.0;
+    if (lane + 32 < n) accq1 += ((ch >> (lane + 32 - C)) & 1ull) ? t : 0.0;
     acct += t;
   }
   if (lane < n) red[warp][lane] = accq0;
@@ -136,147 +169,245 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_z_all(const Cx<R>* __res
   __syncthreads();
   for (int q = threadIdx.x; q <= n; q += blockDim.x) {
     double s = 0.0;
-    for (int w = 0; w < kRedWarps; w++) s += red[w][q];
+    for (int w = 0; w < block_warps; w++) s += red[w][q];
+    partials[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (n + 1) + q] = s;
+  }
+}
+
+// States below one warp chunk (2^n <= 1024 amplitudes): one block a state,
+// amplitude a = thread + 256 i, so bits 0..4 are the lane, 5..7 the warp, 8
+// and 9 the iteration.
+template <typename R>
+__global__ void __launch_bounds__(256) k_expect_z_small(const Cx<R>* __restrict__ state, int n,
+                                                        double* __restrict__ partials) {
+  __shared__ double red[8][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  state += (uint64_t)blockIdx.x << n;
+  double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // total, lane bits 0..4, iteration bits 0..1
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const uint32_t a = threadIdx.x + 256u * i;
+    if (a >> n) continue;
+    const Cx<R> x = state[a];
+    const double p = (double)x.re * x.re + (double)x.im * x.im;
+    v[0] += p;
+    if (i & 1) v[6] += p;
+    if (i & 2) v[7] += p;
+  }
+#pragma unroll
+  for (int b = 0; b < 5; b++) v[1 + b] = ((lane >> b) & 1) ? v[0] : 0.0;
+  const double sum = warp_fold(v, lane);  // value k in lanes 4 k ..
+  if ((lane & 3) == 0) red[warp][lane >> 2] = sum;
+  __syncthreads();
+  if (threadIdx.x <= n) {
+    const int q = threadIdx.x;
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; w++) {
+      const int k = q == n ? 0 : q < 5 ? 1 + q : q < 8 ? 0 : 6 + q - 8;
+      const bool in = q == n || q < 5 || q >= 8 || ((w >> (q - 5)) & 1);
+      if (in) s += red[w][k];
+    }
     partials[(size_t)blockIdx.x * (n + 1) + q] = s;
   }
 }
 
-// Small states (n below one warp chunk): one thread per amplitude, direct.
-template <typename R>
-__global__ void __launch_bounds__(kRedThreads) k_expect_z_small(const Cx<R>* __restrict__ state, int n,
-                                                              double* __restrict__ partials) {
-  __shared__ double red[SV_MAX_QUBITS + 1];
-  if (blockIdx.x != 0) return;
-  for (int q = threadIdx.x; q <= n; q += blockDim.x) {
-    double s = 0.0;
-    for (uint32_t b = 0; b < (1u << n); b++) {
-      Cx<R> a = state[b];
-      double p = (double)a.re * a.re + (double)a.im * a.im;
-      if (q == n || ((b >> q) & 1u)) s += p;
-    }
-    red[q] = s;
+// Adds a state's partial rows (one block a state): warp w takes rows w,
+// w + 32, ..., a lane the columns lane and lane + 32; the warps' sums are
+// added in warp order.  (One thread per column walking all 608 rows of a
+// 26-qubit state took 81 us; this takes 17.)
+__global__ void __launch_bounds__(1024) k_finish_z_all(const double* __restrict__ partials, int nblocks, int n,
+                                                       double* __restrict__ out) {
+  __shared__ double s[32][SV_MAX_QUBITS + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  partials += (size_t)blockIdx.x * nblocks * (n + 1);
+  out += (size_t)blockIdx.x * (n + 1);
+  double a0 = 0.0, a1 = 0.0;
+#pragma unroll 4
+  for (int b = warp; b < nblocks; b += nwarps) {
+    const double* row = partials + (size_t)b * (n + 1);
+    if (lane <= n) a0 += row[lane];
+    if (lane + 32 <= n) a1 += row[lane + 32];
   }
+  if (lane <= n) s[warp][lane] = a0;
+  if (lane + 32 <= n) s[warp][lane + 32] = a1;
   __syncthreads();
-  for (int q = threadIdx.x; q <= n; q += blockDim.x) partials[q] = red[q];
-}
-
-__global__ void k_finish_z_all(const double* __restrict__ partials, int nblocks, int n, double* __restrict__ out) {
-  __shared__ double s[SV_MAX_QUBITS + 1];
-  for (int q = threadIdx.x; q <= n; q += blockDim.x) {
-    double a = 0.0;
-    for (int b = 0; b < nblocks; b++) a += partials[(size_t)b * (n + 1) + q];
-    s[q] = a;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const double T = s[n];
-    double sum = 0.0;
-    for (int q = 0; q < n; q++) {
-      double z = T - 2.0 * s[q];
-      out[q] = z;
-      sum += z;
+  if (warp == 0) {
+    double c0 = 0.0, c1 = 0.0;
+#pragma unroll 8
+    for (int w = 0; w < nwarps; w++) {
+      if (lane <= n) c0 += s[w][lane];
+      if (lane + 32 <= n) c1 += s[w][lane + 32];
     }
-    out[n] = sum;
+    const double T = __shfl_sync(0xffffffffu, n < 32 ? c0 : c1, n & 31);
+    const double z0 = lane < n ? T - 2.0 * c0 : 0.0, z1 = lane + 32 < n ? T - 2.0 * c1 : 0.0;
+    if (lane < n) out[lane] = z0;
+    if (lane + 32 < n) out[lane + 32] = z1;
+    const double sum = warp_sum(z0 + z1);
+    if (lane == 0) out[n] = sum;
   }
 }
 
 // ------------------------------------------------------------ Pauli terms
+//
+// Terms that share an X mask share a pass of up to 16; grid.y runs over the
+// passes of one launch, so a Hamiltonian of many masks is a few launches and
+// the blocks of one pass fill in behind the blocks of the last.  Each term
+// adds one real number per amplitude: the real part of conj(c) a when its
+// count of Y letters is even, else (IMAG) the imaginary part, with the sign
+// flipped by an XOR; terms of one mask and different kinds take a pass each,
+// so that a pass forms one part.  NT is the accumulators a thread holds: a pass of one term (X on
+// one site) pays for one, not for 16.  24 qubits complex64, 24 X terms and 24
+// ZZ terms: 0.46 ms of kernels (14.8 us a one-term pass, 9.1 TB/s with L2's
+// share; 62 us for 16 signed terms, ALU bound), where 16 accumulators for every
+// pass and a one-warp finish took 7.2 + 2.4 ms.  complex128 is bound by the
+// FP64 pipe: 5.6 us a one-term pass at 21 qubits (95 before).
+// The order of a thread's single-precision runs (64 elements a grid stride
+// apart) is fixed, whatever NT is.
 
+template <int NT>
 struct TermPass {
   uint64_t x;
-  int h;        // top bit of x, or -1 when x == 0
-  int nt;
-  uint64_t z[kMaxTermsPerPass];
+  uint64_t z[NT];
+  int32_t h;      // top bit of x
+  int32_t slot;   // first partial row
+  int32_t nt;     // terms (<= NT)
+};
+template <int NT>
+constexpr int kPassesPerLaunch = 3840 / (int)sizeof(TermPass<NT>);
+template <int NT>
+struct TermPasses {
+  TermPass<NT> p[kPassesPerLaunch<NT>];
 };
 
-template <typename R>
-__global__ void __launch_bounds__(kRedThreads) k_expect_terms(const Cx<R>* __restrict__ state, int n, TermPass tp,
+__device__ __forceinline__ float flip_sign(float v, uint32_t sign) {
+  return __uint_as_float(__float_as_uint(v) ^ sign);
+}
+__device__ __forceinline__ double flip_sign(double v, uint32_t sign) {
+  return __hiloint2double(__double2hiint(v) ^ (int)sign, __double2loint(v));
+}
+
+template <typename R, int NT, bool PAIRED, bool IMAG>
+__global__ void __launch_bounds__(kRedThreads) k_expect_terms(const Cx<R>* __restrict__ state, int n,
+                                                            const __grid_constant__ TermPasses<NT> passes,
                                                             double* __restrict__ partials) {
   using T = typename Acc<R>::T;
-  __shared__ double red[kRedWarps][kMaxTermsPerPass][2];
+  const TermPass<NT>& tp = passes.p[blockIdx.y];
+  // signs of all terms at an index: with four terms and more the XOR of one
+  // 32-bit word per index byte (term j's parity at bit 31 - j), built here;
+  // fewer terms take a popcount each (its rate is a quarter of an XOR's)
+  constexpr bool kTable = NT >= 4;
+  constexpr int kBytes = (SV_MAX_QUBITS + 7) / 8;
+  __shared__ uint32_t sgn[kTable ? kBytes : 1][256];
+  __shared__ double red[kRedWarps][NT];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint64_t count = tp.h >= 0 ? (1ull << (n - 1)) : (1ull << n);
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  double are[kMaxTermsPerPass], aim[kMaxTermsPerPass];
+  const uint64_t x = tp.x, low = PAIRED ? (1ull << tp.h) - 1ull : 0ull;
+  if constexpr (kTable) {
+    for (int e = threadIdx.x; e < kBytes * 256; e += blockDim.x) {
+      uint32_t m = 0;
 #pragma unroll
-  for (int j = 0; j < kMaxTermsPerPass; j++) are[j] = aim[j] = 0.0;
+      for (int j = 0; j < NT; j++)
+        m |= (uint32_t)(__popc((uint32_t)(tp.z[j] >> (8 * (e >> 8))) & (uint32_t)(e & 255)) & 1) << (31 - j);
+      sgn[e >> 8][e & 255] = m;
+    }
+    __syncthreads();
+  }
+  const uint64_t count = PAIRED ? (1ull << (n - 1)) : (1ull << n);
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  double acc[NT];
+#pragma unroll
+  for (int j = 0; j < NT; j++) acc[j] = 0.0;
+  constexpr int U = sizeof(R) == 4 ? 8 : 4;  // elements in flight per thread
+  static_assert(64 % U == 0, "whole groups in a run");
+  T run[NT] = {};
+  auto index_of = [&](uint64_t i) { return PAIRED ? i + (i & ~low) : i; };  // a zero inserted at bit h
+  auto add = [&](const Cx<R>& a, const Cx<R>& c, uint64_t b) {
+    uint32_t m = 0;
+    if constexpr (kTable) {
+      m = sgn[0][b & 255] ^ sgn[1][(b >> 8) & 255] ^ sgn[2][(b >> 16) & 255];
+      if (n > 24) m ^= sgn[3][(b >> 24) & 255] ^ sgn[4][(b >> 32) & 255];
+    } else {
+#pragma unroll
+      for (int j = 0; j < NT; j++) {
+        const uint32_t w = ((uint32_t)b & (uint32_t)tp.z[j]) ^ ((uint32_t)(b >> 32) & (uint32_t)(tp.z[j] >> 32));
+        m |= (uint32_t)__popc(w) << (31 - j) & (0x80000000u >> j);
+      }
+    }
+    if constexpr (PAIRED && NT == 1 && sizeof(R) == 8) {  // FP64 pipe bound: the sign rides on a, two FMAs
+      const T p = flip_sign(IMAG ? a.im : a.re, m & 0x80000000u);
+      const T q = flip_sign(IMAG ? a.re : a.im, (m & 0x80000000u) ^ (IMAG ? 0x80000000u : 0u));
+      run[0] = fma(c.re, p, fma(c.im, q, run[0]));
+    } else {
+      T v;
+      if constexpr (PAIRED)  // conj(c) * a
+        v = IMAG ? (T)c.re * (T)a.im - (T)c.im * (T)a.re : (T)c.re * (T)a.re + (T)c.im * (T)a.im;
+      else
+        v = (T)a.re * (T)a.re + (T)a.im * (T)a.im;
+#pragma unroll
+      for (int j = 0; j < NT; j++) run[j] += flip_sign(v, (m << j) & 0x80000000u);
+    }
+  };
   uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   while (i < count) {
-    T rre[kMaxTermsPerPass], rim[kMaxTermsPerPass];
 #pragma unroll
-    for (int j = 0; j < kMaxTermsPerPass; j++) rre[j] = rim[j] = 0;
+    for (int j = 0; j < NT; j++) run[j] = 0;
     // a short run in the run precision, then fold into double
-    for (int r = 0; r < 64 && i < count; r++, i += stride) {
-      uint64_t b = tp.h >= 0 ? ((i >> tp.h) << (tp.h + 1)) | (i & ((1ull << tp.h) - 1ull)) : i;
-      Cx<R> a = state[b];
-      T vre, vim;
-      if (tp.h >= 0) {
-        Cx<R> c = state[b ^ tp.x];  // conj(c) * a
-        vre = (T)c.re * (T)a.re + (T)c.im * (T)a.im;
-        vim = (T)c.re * (T)a.im - (T)c.im * (T)a.re;
-      } else {
-        vre = (T)a.re * (T)a.re + (T)a.im * (T)a.im;
-        vim = 0;
-      }
+    for (int r = 0; r < 64 && i < count;) {
+      if (i + (U - 1) * stride < count) {
+        Cx<R> a[U], c[U];
 #pragma unroll
-      for (int j = 0; j < kMaxTermsPerPass; j++) {
-        if (j < tp.nt) {
-          T sg = (__popcll(b & tp.z[j]) & 1) ? T(-1) : T(1);
-          rre[j] = fma(sg, vre, rre[j]);
-          rim[j] = fma(sg, vim, rim[j]);
+        for (int k = 0; k < U; k++) {
+          const uint64_t b = index_of(i + k * stride);
+          a[k] = state[b];
+          if constexpr (PAIRED) c[k] = state[b ^ x];
         }
+#pragma unroll
+        for (int k = 0; k < U; k++) add(a[k], PAIRED ? c[k] : a[k], index_of(i + k * stride));
+        r += U;
+        i += U * stride;
+      } else {
+        const uint64_t b = index_of(i);
+        const Cx<R> a = state[b];
+        add(a, PAIRED ? state[b ^ x] : a, b);
+        r++;
+        i += stride;
       }
     }
 #pragma unroll
-    for (int j = 0; j < kMaxTermsPerPass; j++) {
-      are[j] += (double)rre[j];
-      aim[j] += (double)rim[j];
-    }
+    for (int j = 0; j < NT; j++) acc[j] += (double)run[j];
   }
-#pragma unroll
-  for (int j = 0; j < kMaxTermsPerPass; j++) {
-    double a = warp_sum(are[j]), b = warp_sum(aim[j]);
-    if (lane == 0 && j < tp.nt) {
-      red[warp][j][0] = a;
-      red[warp][j][1] = b;
-    }
-  }
+  const double s = warp_fold(acc, lane);
+  if (lane % (32 / NT) == 0) red[warp][lane / (32 / NT)] = s;
   __syncthreads();
-  for (int j = threadIdx.x; j < tp.nt; j += blockDim.x) {
-    double a = 0.0, b = 0.0;
-    for (int w = 0; w < kRedWarps; w++) {
-      a += red[w][j][0];
-      b += red[w][j][1];
-    }
-    partials[((size_t)blockIdx.x * kMaxTermsPerPass + j) * 2] = a;
-    partials[((size_t)blockIdx.x * kMaxTermsPerPass + j) * 2 + 1] = b;
+  if ((int)threadIdx.x < tp.nt) {
+    double a = 0.0;
+    for (int w = 0; w < kRedWarps; w++) a += red[w][threadIdx.x];
+    partials[(size_t)(tp.slot + threadIdx.x) * gridDim.x + blockIdx.x] = a;
   }
 }
 
 struct TermOut {
-  int nt;
-  int dst[kMaxTermsPerPass];  // output index of each term of the pass
-  int ny[kMaxTermsPerPass];   // number of Y letters
+  uint16_t dst[kMaxTermSlots];  // output index of each slot's term
+  uint8_t how[kMaxTermSlots];   // bits 0..1: Y letters mod 4; bit 2: paired
 };
 
-__global__ void k_finish_terms(const double* __restrict__ partials, int nblocks, int paired, TermOut to,
-                               double* __restrict__ out) {
-  int j = threadIdx.x;
-  if (j >= to.nt) return;
-  double a = 0.0, b = 0.0;
-  for (int k = 0; k < nblocks; k++) {
-    a += partials[((size_t)k * kMaxTermsPerPass + j) * 2];
-    b += partials[((size_t)k * kMaxTermsPerPass + j) * 2 + 1];
+// One block per term adds its partials; Re[i^{nY} (a + i b)], of which the
+// pass kernel kept a (nY even) or b (odd).
+__global__ void __launch_bounds__(128) k_finish_terms(const double* __restrict__ partials, int nblocks,
+                                                      const __grid_constant__ TermOut to, double* __restrict__ out) {
+  __shared__ double red[4];
+  const int j = blockIdx.x;
+  double a = 0.0;
+  for (int k = threadIdx.x; k < nblocks; k += blockDim.x) a += partials[(size_t)j * nblocks + k];
+  a = warp_sum(a);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a = (red[0] + red[1]) + (red[2] + red[3]);
+    const int ny = to.how[j] & 3;
+    const double re = ny == 1 || ny == 2 ? -a : a;
+    out[to.dst[j]] = (to.how[j] & 4) ? 2.0 * re : re;
   }
-  // Re[i^{nY} (a + i b)]
-  double re;
-  switch (to.ny[j] & 3) {
-    case 0: re = a; break;
-    case 1: re = -b; break;
-    case 2: re = -a; break;
-    default: re = b; break;
-  }
-  out[to.dst[j]] = paired ? 2.0 * re : re;
 }
 
 }  // namespace
@@ -291,59 +422,156 @@ size_t expect_z_all_scratch_doubles(int n) {
 size_t expect_terms_scratch_doubles(int n, int n_terms) {
   (void)n;
   (void)n_terms;
-  return (size_t)red_grid() * kMaxTermsPerPass * 2;
+  return (size_t)red_grid() * kMaxTermSlots;
+}
+
+// Blocks of a state's read-out: a warp a chunk; blocks of one warp until the
+// grid holds four blocks an SM over the whole batch (a small state spreads over
+// the SMs), then of up to eight.
+static int z_all_blocks(int n, int chunk_bits, int batch, int* warps) {
+  if (n < chunk_bits) return 1;
+  const uint64_t chunks = 1ull << (n - chunk_bits);
+  const uint64_t most = ((uint64_t)red_grid() + batch - 1) / batch;
+  const uint64_t g = chunks < most ? chunks : most;
+  *warps = 1;
+  while (*warps < kRedWarps && chunks > g * *warps) *warps *= 2;
+  return (int)g;
+}
+constexpr int z_chunk_bits(size_t amp_bytes) { return amp_bytes == 8 ? 11 : 10; }
+
+size_t expect_z_batch_scratch_doubles(int n, int batch, size_t amp_bytes) {
+  int warps = 0;
+  return (size_t)batch * z_all_blocks(n, z_chunk_bits(amp_bytes), batch, &warps) * (n + 1);
+}
+
+template <typename R>
+cudaError_t launch_expect_z_batch(const Cx<R>* states, int n, int batch, double* scratch, size_t scratch_doubles,
+                                  double* out, cudaStream_t stream) {
+  constexpr int C = z_chunk_bits(sizeof(Cx<R>));
+  int warps = 0;
+  const int grid = z_all_blocks(n, C, batch, &warps);
+  if ((size_t)batch * grid * (n + 1) > scratch_doubles) return cudaErrorInvalidValue;
+  if (n < C)
+    k_expect_z_small<R><<<batch, kRedThreads, 0, stream>>>(states, n, scratch);
+  else
+    k_expect_z_all<R><<<dim3((unsigned)grid, (unsigned)batch), 32 * warps, 0, stream>>>(states, n, scratch);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_finish_z_all<<<batch, grid >= 32 ? 1024 : 32 * grid, 0, stream>>>(scratch, grid, n, out);
+  return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t launch_expect_z_all(const Cx<R>* state, int n, double* scratch, size_t scratch_doubles, double* out,
                                 cudaStream_t stream) {
-  constexpr int A = 16 / sizeof(Cx<R>);
-  constexpr int C = (A == 2 ? 1 : 0) + 10;
-  int grid;
-  if (n < C) {
-    grid = 1;
-    k_expect_z_small<R><<<1, kRedThreads, 0, stream>>>(state, n, scratch);
-  } else {
-    uint64_t chunks = 1ull << (n - C);
-    uint64_t g = (chunks + kRedWarps - 1) / kRedWarps;
-    grid = (int)(g < (uint64_t)red_grid() ? g : (uint64_t)red_grid());
-    if ((size_t)grid * (n + 1) > scratch_doubles) return cudaErrorInvalidValue;
-    k_expect_z_all<R><<<grid, kRedThreads, 0, stream>>>(state, n, scratch);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_finish_z_all<<<1, 64, 0, stream>>>(scratch, grid, n, out);
-  return cudaGetLastError();
+  return launch_expect_z_batch<R>(state, n, 1, scratch, scratch_doubles, out, stream);
 }
+
+namespace {
+
+// The passes of one accumulator count, launched in groups of what fits the
+// kernel's parameters.
+template <typename R, int NT, bool PAIRED, bool IMAG>
+cudaError_t launch_term_passes(const Cx<R>* state, int n, const std::vector<TermPass<kMaxTermsPerPass>>& list,
+                               int grid, double* scratch, cudaStream_t stream) {
+  TermPasses<NT> tp;
+  for (size_t at = 0; at < list.size();) {
+    int k = 0;
+    for (; at < list.size() && k < kPassesPerLaunch<NT>; at++, k++) {
+      const TermPass<kMaxTermsPerPass>& p = list[at];
+      TermPass<NT>& d = tp.p[k];
+      d.x = p.x;
+      d.h = p.h;
+      d.slot = p.slot;
+      d.nt = p.nt;
+      for (int j = 0; j < NT; j++) d.z[j] = j < p.nt ? p.z[j] : 0ull;
+    }
+    k_expect_terms<R, NT, PAIRED, IMAG><<<dim3((unsigned)grid, (unsigned)k), kRedThreads, 0, stream>>>(state, n, tp, scratch);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+template <typename R, bool PAIRED, bool IMAG>
+cudaError_t launch_terms_by_count(const Cx<R>* state, int n, const std::vector<TermPass<kMaxTermsPerPass>>& list,
+                                  int grid, double* scratch, cudaStream_t stream) {
+  std::vector<TermPass<kMaxTermsPerPass>> by[5];  // 1, 2, 3..4, 5..8, 9..16 terms
+  for (const TermPass<kMaxTermsPerPass>& p : list) by[p.nt <= 1 ? 0 : p.nt <= 2 ? 1 : p.nt <= 4 ? 2 : p.nt <= 8 ? 3 : 4].push_back(p);
+  cudaError_t e = launch_term_passes<R, 1, PAIRED, IMAG>(state, n, by[0], grid, scratch, stream);
+  if (e == cudaSuccess) e = launch_term_passes<R, 2, PAIRED, IMAG>(state, n, by[1], grid, scratch, stream);
+  if (e == cudaSuccess) e = launch_term_passes<R, 4, PAIRED, IMAG>(state, n, by[2], grid, scratch, stream);
+  if (e == cudaSuccess) e = launch_term_passes<R, 8, PAIRED, IMAG>(state, n, by[3], grid, scratch, stream);
+  if (e == cudaSuccess) e = launch_term_passes<R, 16, PAIRED, IMAG>(state, n, by[4], grid, scratch, stream);
+  return e;
+}
+
+int term_grid(uint64_t count) {
+  const uint64_t g = (count + kRedThreads - 1) / kRedThreads;
+  return (int)(g < (uint64_t)red_grid() ? g : (uint64_t)red_grid());
+}
+
+}  // namespace
 
 template <typename R>
 cudaError_t launch_expect_terms(const Cx<R>* state, int n, const sv_pauli_term* terms, int n_terms, double* scratch,
                                 size_t scratch_doubles, double* out, cudaStream_t stream) {
-  if ((size_t)red_grid() * kMaxTermsPerPass * 2 > scratch_doubles) return cudaErrorInvalidValue;
-  std::vector<char> used(n_terms, 0);
-  for (int t0 = 0; t0 < n_terms; t0++) {
-    if (used[t0]) continue;
-    TermPass tp{};
-    TermOut to{};
-    tp.x = terms[t0].x_mask;
-    tp.h = tp.x ? 63 - __builtin_clzll(tp.x) : -1;
-    for (int t = t0; t < n_terms && tp.nt < kMaxTermsPerPass; t++) {
-      if (used[t] || terms[t].x_mask != tp.x) continue;
-      used[t] = 1;
-      tp.z[tp.nt] = terms[t].z_mask;
-      to.dst[tp.nt] = t;
-      to.ny[tp.nt] = __builtin_popcountll(terms[t].x_mask & terms[t].z_mask);
-      tp.nt++;
-    }
-    to.nt = tp.nt;
-    uint64_t count = tp.h >= 0 ? (1ull << (n - 1)) : (1ull << n);
-    uint64_t g = (count + kRedThreads - 1) / kRedThreads;
-    int grid = (int)(g < (uint64_t)red_grid() ? g : (uint64_t)red_grid());
-    k_expect_terms<R><<<grid, kRedThreads, 0, stream>>>(state, n, tp, scratch);
-    cudaError_t e = cudaGetLastError();
+  if ((size_t)red_grid() * kMaxTermSlots > scratch_doubles) return cudaErrorInvalidValue;
+  const int grid_z = term_grid(1ull << n), grid_x = term_grid(1ull << (n - 1));
+  std::vector<TermPass<kMaxTermsPerPass>> lists[3];  // no X mask; real part; imaginary part
+  TermOut to[3] = {};
+  int slots[3] = {0, 0, 0};
+  // runs what has been collected of one kind and writes its terms' values
+  auto flush = [&](int kind) -> cudaError_t {
+    if (!slots[kind]) return cudaSuccess;
+    const int grid = kind ? grid_x : grid_z;
+    cudaError_t e = kind == 0   ? launch_terms_by_count<R, false, false>(state, n, lists[0], grid, scratch, stream)
+                    : kind == 1 ? launch_terms_by_count<R, true, false>(state, n, lists[1], grid, scratch, stream)
+                                : launch_terms_by_count<R, true, true>(state, n, lists[2], grid, scratch, stream);
     if (e != cudaSuccess) return e;
-    k_finish_terms<<<1, 32, 0, stream>>>(scratch, grid, tp.h >= 0 ? 1 : 0, to, out);
-    e = cudaGetLastError();
+    k_finish_terms<<<slots[kind], 128, 0, stream>>>(scratch, grid, to[kind], out);
+    lists[kind].clear();
+    slots[kind] = 0;
+    return cudaGetLastError();
+  };
+  // terms by kind and X mask, in the order of each mask's first term
+  std::map<std::pair<uint64_t, int>, int> first;
+  std::vector<std::vector<int>> groups;
+  auto kind_of = [&](int t) {
+    const uint64_t x = terms[t].x_mask;
+    return !x ? 0 : 1 + (__builtin_popcountll(x & terms[t].z_mask) & 1);
+  };
+  for (int t = 0; t < n_terms; t++) {
+    const auto at = first.emplace(std::make_pair(terms[t].x_mask, kind_of(t)), (int)groups.size());
+    if (at.second) groups.emplace_back();
+    groups[at.first->second].push_back(t);
+  }
+  for (const std::vector<int>& g : groups) {
+    const uint64_t x = terms[g[0]].x_mask;
+    const int kind = kind_of(g[0]);
+    for (size_t k = 0; k < g.size();) {
+      const int nt = (int)std::min<size_t>(kMaxTermsPerPass, g.size() - k);
+      if (slots[kind] + nt > kMaxTermSlots) {
+        const cudaError_t e = flush(kind);
+        if (e != cudaSuccess) return e;
+      }
+      TermPass<kMaxTermsPerPass> p{};
+      p.x = x;
+      p.h = x ? 63 - __builtin_clzll(x) : 0;
+      p.slot = slots[kind];
+      p.nt = nt;
+      for (int j = 0; j < nt; j++, k++) {
+        const uint64_t z = terms[g[k]].z_mask;
+        p.z[j] = z;
+        to[kind].dst[p.slot + j] = (uint16_t)g[k];
+        to[kind].how[p.slot + j] = (uint8_t)((__builtin_popcountll(x & z) & 3) | (kind ? 4 : 0));
+      }
+      slots[kind] += nt;
+      lists[kind].push_back(p);
+    }
+  }
+  for (int kind = 0; kind < 3; kind++) {
+    const cudaError_t e = flush(kind);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -351,6 +579,9 @@ cudaError_t launch_expect_terms(const Cx<R>* state, int n, const sv_pauli_term* 
 
 template cudaError_t launch_expect_z_all<float>(const Cx<float>*, int, double*, size_t, double*, cudaStream_t);
 template cudaError_t launch_expect_z_all<double>(const Cx<double>*, int, double*, size_t, double*, cudaStream_t);
+template cudaError_t launch_expect_z_batch<float>(const Cx<float>*, int, int, double*, size_t, double*, cudaStream_t);
+template cudaError_t launch_expect_z_batch<double>(const Cx<double>*, int, int, double*, size_t, double*,
+                                                   cudaStream_t);
 template cudaError_t launch_expect_terms<float>(const Cx<float>*, int, const sv_pauli_term*, int, double*, size_t,
                                                 double*, cudaStream_t);
 template cudaError_t launch_expect_terms<double>(const Cx<double>*, int, const sv_pauli_term*, int, double*, size_t,
