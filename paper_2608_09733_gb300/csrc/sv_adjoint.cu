@@ -523,14 +523,19 @@ __global__ void k_build_tables(const double* __restrict__ params, int npar, int 
 }
 
 // out[b, p] = sum of g[b, pidx] over the parameterised gates pidx bound to
-// slot p (in gate order, so the sums do not depend on scheduling).
-__global__ void k_scatter_grad(const double* __restrict__ g, int batch, int ngrad, const int* __restrict__ slot,
-                               int npar, double* __restrict__ out) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= batch) return;
-  double* o = out + (size_t)b * npar;
-  for (int p = 0; p < npar; p++) o[p] = 0.0;
-  for (int k = 0; k < ngrad; k++) o[slot[k]] += g[(size_t)b * ngrad + k];
+// slot p, in gate order (so the sums do not depend on scheduling): by_slot
+// lists the gates of slot 0, slot 1, ...; slot p's are at first[p] ..
+// first[p + 1] - 1.  A thread per (state, slot): one thread per state walking
+// every gate took 125 us for 64 states of 400 parameters.
+__global__ void k_scatter_grad(const double* __restrict__ g, int batch, int ngrad, const int* __restrict__ first,
+                               const int* __restrict__ by_slot, int npar, double* __restrict__ out) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)batch * npar) return;
+  const int p = (int)(i % npar);
+  const double* row = g + (i / npar) * ngrad;
+  double s = 0.0;
+  for (int k = first[p]; k < first[p + 1]; k++) s += row[by_slot[k]];
+  out[i] = s;
 }
 
 }  // namespace
@@ -544,10 +549,11 @@ cudaError_t launch_build_tables(const double* params, int npar, int batch, const
   return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_grad(const double* g, int batch, int ngrad, const int* slot, int npar, double* out,
-                                cudaStream_t stream) {
-  if (batch == 0 || npar == 0) return cudaSuccess;
-  k_scatter_grad<<<(batch + 127) / 128, 128, 0, stream>>>(g, batch, ngrad, slot, npar, out);
+cudaError_t launch_scatter_grad(const double* g, int batch, int ngrad, const int* first, const int* by_slot, int npar,
+                                double* out, cudaStream_t stream) {
+  const long long n = (long long)batch * npar;
+  if (n == 0) return cudaSuccess;
+  k_scatter_grad<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(g, batch, ngrad, first, by_slot, npar, out);
   return cudaGetLastError();
 }
 

@@ -50,9 +50,10 @@ struct TableGate {
 template <typename R>
 cudaError_t launch_build_tables(const double* params, int npar, int batch, const TableGate* gates, int ngates,
                                 Cx<R>* table, cudaStream_t stream);
-// out[b * npar + p] = sum over k with slot[k] == p of g[b * ngrad + k] (device).
-cudaError_t launch_scatter_grad(const double* g, int batch, int ngrad, const int* slot, int npar, double* out,
-                                cudaStream_t stream);
+// out[b * npar + p] = sum over k in by_slot[first[p] .. first[p + 1]) of
+// g[b * ngrad + k] (device arrays; first has npar + 1 entries).
+cudaError_t launch_scatter_grad(const double* g, int batch, int ngrad, const int* first, const int* by_slot, int npar,
+                                double* out, cudaStream_t stream);
 // ----------------------------------------------------------------- compiled batched kernels (sv_jit.cpp)
 // The kernel source of one batched program (every phase and op a constant).
 template <typename R>

@@ -526,18 +526,23 @@ void run_adjoint(int n, sv_dtype dtype, const sv_gate* gates, size_t ng, const d
   double* gout = (double*)scratch_buffer(stream, "adj_gout", sizeof(double) * (size_t)batch * std::max(npg, 1));
   double* dots = (double*)scratch_buffer(stream, "adj_dot", sizeof(double) * batch_dot_scratch_doubles(batch));
   double* vout = (double*)scratch_buffer(stream, "adj_val", sizeof(double) * batch);
-  int* dslot = nullptr;
+  int* dslots = nullptr;  // first[npar + 1], by_slot[npg]: the gates of each slot, in gate order
   if (dev) {  // the gate list and slots go up (small); the matrices are built where the parameters are
     TableGate* dg = (TableGate*)scratch_buffer(stream, "adj_tgates", sizeof(TableGate) * std::max<size_t>(npg, 1));
-    dslot = (int*)scratch_buffer(stream, "adj_pslot", sizeof(int) * std::max<size_t>(npg, 1));
+    const size_t nslots = (size_t)npar + 1 + npg;
+    dslots = (int*)scratch_buffer(stream, "adj_pslot", sizeof(int) * nslots);
     if (npg) {
-      Pinned& pin = pinned_buffer(stream, "adj_tgates", sizeof(TableGate) * npg + sizeof(int) * npg);
+      Pinned& pin = pinned_buffer(stream, "adj_tgates", sizeof(TableGate) * npg + sizeof(int) * nslots);
       std::memcpy(pin.p, tgates.data(), sizeof(TableGate) * npg);
-      std::memcpy((char*)pin.p + sizeof(TableGate) * npg, pslot.data(), sizeof(int) * npg);
+      int* first = (int*)((char*)pin.p + sizeof(TableGate) * npg);
+      int* by_slot = first + npar + 1;
+      std::fill(first, first + npar + 1, 0);
+      for (int sl : pslot) first[sl + 1]++;
+      for (int p = 0; p < npar; p++) first[p + 1] += first[p];
+      std::vector<int> at(first, first + npar);
+      for (int k = 0; k < npg; k++) by_slot[at[pslot[k]]++] = k;
       cuda_check(cudaMemcpyAsync(dg, pin.p, sizeof(TableGate) * npg, cudaMemcpyHostToDevice, stream), "gate list");
-      cuda_check(cudaMemcpyAsync(dslot, (char*)pin.p + sizeof(TableGate) * npg, sizeof(int) * npg,
-                                 cudaMemcpyHostToDevice, stream),
-                 "slot list");
+      cuda_check(cudaMemcpyAsync(dslots, first, sizeof(int) * nslots, cudaMemcpyHostToDevice, stream), "slot list");
       cuda_check(cudaEventRecord(pin.ready, stream), "cudaEventRecord");
     }
     cuda_check(launch_build_tables<R>(params, npar, batch, dg, npg, dtab, stream), "gate tables");
@@ -578,12 +583,10 @@ void run_adjoint(int n, sv_dtype dtype, const sv_gate* gates, size_t ng, const d
   // ---- forward-only: <Z_q> of every state
   if (out_z) {
     const size_t zn = (size_t)n + 1;
-    double* zscr = (double*)scratch_buffer(stream, "adj_zscratch", sizeof(double) * expect_z_all_scratch_doubles(n));
+    const size_t zsd = expect_z_batch_scratch_doubles(n, batch, sizeof(Cx<R>));
+    double* zscr = (double*)scratch_buffer(stream, "adj_zscratch", sizeof(double) * zsd);
     double* zdev = dev ? out_z : (double*)scratch_buffer(stream, "adj_zout", sizeof(double) * zn * batch);
-    for (int b = 0; b < batch; b++)
-      cuda_check(launch_expect_z_all<R>(psi + (size_t)b * N, n, zscr, expect_z_all_scratch_doubles(n),
-                                        zdev + (size_t)b * zn, stream),
-                 "per-state <Z>");
+    cuda_check(launch_expect_z_batch<R>(psi, n, batch, zscr, zsd, zdev, stream), "per-state <Z>");
     if (dev) return;
     cuda_check(cudaMemcpyAsync(out_z, zdev, sizeof(double) * zn * batch, cudaMemcpyDeviceToHost, stream),
                "<Z> copy");
@@ -650,7 +653,8 @@ void run_adjoint(int n, sv_dtype dtype, const sv_gate* gates, size_t ng, const d
   if (npg) cuda_check(launch_grad_finish(gscr, batch, npg, grid_x, gout, stream), "gradient reduce");
   if (dev) {  // slots shared by several gates add up, on the device
     if (npg) {
-      cuda_check(launch_scatter_grad(gout, batch, npg, dslot, npar, out_grad, stream), "gradient scatter");
+      cuda_check(launch_scatter_grad(gout, batch, npg, dslots, dslots + npar + 1, npar, out_grad,
+                                     stream), "gradient scatter");
     } else if (npar) {
       cuda_check(cudaMemsetAsync(out_grad, 0, sizeof(double) * (size_t)batch * npar, stream), "gradient clear");
     }
