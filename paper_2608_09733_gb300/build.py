@@ -22,13 +22,13 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libsv.so")
 
 SOURCES = ["sv_plan.cpp", "sv_program.cpp", "sv_api.cpp", "sv_adjoint_host.cpp", "sv_serve.cpp", "sv_jit.cpp",
-           "sv_sweep.cu", "sv_reduce.cu", "sv_adjoint.cu", "sv_noalloc.cu", "sv_sample.cu",
+           "sv_sweep.cu", "sv_lane.cu", "sv_reduce.cu", "sv_adjoint.cu", "sv_noalloc.cu", "sv_sample.cu",
            "sv_hostcopy.cu"]
 # Device headers the run-time compiled pass kernels include (sv_jit.cpp): their
 # text is embedded in the library, so a kernel compiled at run time is built
 # from the same code as the library's own pass kernel.
 JIT_HEADERS = ["sv_prog_layout.h", "sv_pass_ops.cuh", "sv_tma_pass.cuh", "sv_batch_layout.h", "sv_batch_ops.cuh"]
-HEADERS = ["sv_internal.h", "sv_adjoint.h"] + JIT_HEADERS
+HEADERS = ["sv_internal.h", "sv_adjoint.h", "sv_stage.cuh"] + JIT_HEADERS
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "--expt-relaxed-constexpr", "-I" + os.path.join(ROOT, "include"), "-I" + OUT]
@@ -58,7 +58,7 @@ def _stamp(extra=()) -> str:
 
 # Sources that decide what the pass kernel does (the kernel, the program
 # builder, the planner and the shared structures).
-SWEEP_SOURCES = ["sv_sweep.cu", "sv_program.cpp", "sv_plan.cpp", "sv_internal.h", "sv_jit.cpp", "sv_prog_layout.h",
+SWEEP_SOURCES = ["sv_sweep.cu", "sv_lane.cu", "sv_stage.cuh", "sv_program.cpp", "sv_plan.cpp", "sv_internal.h", "sv_jit.cpp", "sv_prog_layout.h",
                  "sv_pass_ops.cuh", "sv_tma_pass.cuh"]
 
 

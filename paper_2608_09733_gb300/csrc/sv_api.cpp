@@ -236,13 +236,13 @@ std::mutex g_compiled_mu;
 std::list<std::shared_ptr<const Compiled>> g_compiled;  // most recent first
 
 std::vector<unsigned char> circuit_key(int n, sv_dtype dtype, const sv_gate* gates, size_t ng, const double* pv,
-                                       size_t npv, const sv_exec_opts& opts) {
+                                       size_t npv, const sv_exec_opts& opts, bool lane) {
   std::vector<unsigned char> k;
   auto put = [&](const void* p, size_t b) {
     const unsigned char* c = (const unsigned char*)p;
     k.insert(k.end(), c, c + b);
   };
-  const int32_t hdr[2] = {n, (int32_t)dtype};
+  const int32_t hdr[3] = {n, (int32_t)dtype, lane ? 1 : 0};
   put(hdr, sizeof(hdr));
   put(&opts, sizeof(opts));
   put(&ng, sizeof(ng));
@@ -261,7 +261,8 @@ std::vector<unsigned char> circuit_key(int n, sv_dtype dtype, const sv_gate* gat
 
 std::shared_ptr<const Compiled> compiled_circuit(int n, sv_dtype dtype, const sv_gate* gates, size_t ng,
                                                  const double* pv, size_t npv, const sv_exec_opts& opts) {
-  std::vector<unsigned char> key = circuit_key(n, dtype, gates, ng, pv, npv, opts);
+  const bool lane = lane_sizes(n, opts) && lane_pass_available();
+  std::vector<unsigned char> key = circuit_key(n, dtype, gates, ng, pv, npv, opts, lane);
   {
     std::lock_guard<std::mutex> lk(g_compiled_mu);
     for (auto it = g_compiled.begin(); it != g_compiled.end(); ++it)
@@ -272,7 +273,7 @@ std::shared_ptr<const Compiled> compiled_circuit(int n, sv_dtype dtype, const sv
         return c;
       }
   }
-  Plan plan = make_plan(n, dtype, gates, ng, pv, npv, opts);
+  Plan plan = make_plan(n, dtype, gates, ng, pv, npv, opts, 0, lane);
   auto c = std::make_shared<Compiled>();
   c->n = n;
   if (dtype == SV_C64) {
@@ -474,7 +475,8 @@ sv_status sv_plan_info(int n_qubits, sv_dtype dtype, const sv_gate* gates, size_
                        const double* param_values, size_t n_param_values, const sv_exec_opts* opts,
                        int* out_blocks, int* out_sweeps, int* block_starts) {
   return guarded([&] {
-    Plan plan = make_plan(n_qubits, dtype, gates, n_gates, param_values, n_param_values, opts_of(opts));
+    const sv_exec_opts o = opts_of(opts);
+    Plan plan = make_plan(n_qubits, dtype, gates, n_gates, param_values, n_param_values, o, 0, lane_sizes(n_qubits, o));
     if (std::getenv("SV_DEBUG_PLAN")) {  // print the device programs (host only)
       std::unique_ptr<SweepProgram<float>> pf(new SweepProgram<float>());
       for (const Sweep& sw : plan.sweeps) build_program<float>(plan, sw, *pf);

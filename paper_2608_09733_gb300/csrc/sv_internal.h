@@ -43,6 +43,11 @@ struct Plan {
   std::vector<LOp> ops;
   std::vector<int> block_starts;  // first gate of each op (fusion blocks) + n_gates
   std::vector<Sweep> sweeps;
+  bool lane = false;        // passes of the cluster kernel (sv_lane.cu): tiles of up to 2^14 amplitudes
+  // phase tables are carried across bit flips and swaps (permuted) instead of
+  // applied before them; not for the packed and session programs, whose
+  // rounding stays as it is
+  bool carry_flips = false;
 };
 
 // Errors carry a status and a message up to the C ABI.
@@ -101,7 +106,9 @@ void classify(LOp& op);
 std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_q, int low_q, int coef_pool,
                                    int ops_per_pass);
 Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, const double* param_values,
-               size_t n_param_values, const sv_exec_opts& opts, int tile_q_override = 0);
+               size_t n_param_values, const sv_exec_opts& opts, int tile_q_override = 0, bool lane = false);
+// Whether a state of this size with these options takes the cluster pass.
+bool lane_sizes(int n, const sv_exec_opts& opts);
 double op_cost(const LOp& op);
 int tile_qubits_for(sv_dtype dtype, int n);
 int low_qubits_for(sv_dtype dtype);
@@ -132,6 +139,12 @@ struct JitKernel;
 template <typename R>
 cudaError_t launch_sweep(Cx<R>* state, const SweepProgram<R>& prog, cudaStream_t stream,
                          const char** kernel = nullptr, const JitKernel* jit = nullptr);
+// The cluster pass of small states (sv_lane.cu); whether the current device
+// takes it now (clusters of 16 CTAs, which a live serving session's resident
+// CTAs could keep waiting, so not beside one).
+template <typename R>
+cudaError_t launch_lane_pass(Cx<R>* state, const SweepProgram<R>& prog, cudaStream_t stream);
+bool lane_pass_available();
 template <typename R>
 cudaError_t launch_init_basis(Cx<R>* state, int n, uint64_t index, cudaStream_t stream);
 // One CTA per small request (whole state in shared memory): request b runs

@@ -561,8 +561,20 @@ static void defer_diagonals(const std::vector<LOp>& ops, std::vector<Sweep>& sw,
   }
 }
 
+// States of up to four cluster tiles (2^14 amplitudes each) take the cluster
+// pass: a tile spread over a cluster's SMs, an amplitude a lane.  At 17 qubits
+// the eight clusters no longer fit beside each other and the one-CTA tiles,
+// 16 of them by then, are faster (complex64, U3 + CNOT ladder of depth 22:
+// 15 qubits 430 against 461 us, 16 qubits 472 against 465 but 287 against 456
+// on random two-qubit matrices, 17 qubits 840 against 552).  Below five
+// qubits there is no warp to fill.  An explicit tile width or cap of
+// operations per pass keeps its own kernel.
+bool lane_sizes(int n, const sv_exec_opts& opts) {
+  return n >= 5 && n <= 16 && opts.tile_qubits == 0 && opts.ops_per_pass == 0;
+}
+
 Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, const double* param_values,
-               size_t n_param_values, const sv_exec_opts& opts, int tile_q_override) {
+               size_t n_param_values, const sv_exec_opts& opts, int tile_q_override, bool lane) {
   const int fuse_max_k = opts.fuse_max_k;
   if (opts.block_mode != SV_BLOCK_AUTO && opts.block_mode != SV_BLOCK_DENSE) fail(SV_ERR_INVALID, "unknown block_mode");
   if (opts.ops_per_pass < 0) fail(SV_ERR_INVALID, "ops_per_pass must be >= 0");
@@ -576,6 +588,8 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
   validate_gates(n, gates, n_gates, n_param_values);
   Plan p;
   p.n = n;
+  p.lane = lane;
+  p.carry_flips = tile_q_override == 0;
   if (fuse_max_k >= 2) {
     p.ops = fuse_greedy(n, gates, n_gates, param_values, fuse_max_k, &p.block_starts,
                         opts.block_mode == SV_BLOCK_DENSE);
@@ -605,6 +619,7 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
   drop_identities(p.ops);
   int pool = dtype == SV_C64 ? SweepProgram<float>::kPool : SweepProgram<double>::kPool;
   const int tile_q = tile_q_override > 0 ? tile_q_override
+                     : lane              ? std::min(n, kMaxTileQ)
                      : opts.tile_qubits > 0 ? std::min(opts.tile_qubits, n)
                                             : tile_qubits_for(dtype, n);
   const int max_ops = opts.ops_per_pass > 0 ? std::min(opts.ops_per_pass, kMaxOps) : kMaxOps;

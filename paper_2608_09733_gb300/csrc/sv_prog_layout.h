@@ -119,7 +119,8 @@ struct Cx {
 struct ProgramHeader {
   int32_t n, m, L, nops;
   int32_t ncoef, nphases;
-  int32_t rq, pad;  // register qubits of the register phases (4 or 5)
+  int32_t rq;       // register qubits of the register phases (4 or 5)
+  int32_t lane;     // 1: a program of the cluster pass (sv_lane.cu), whose register qubits are the lane
   int8_t tq[16];
 };
 

@@ -69,8 +69,9 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
   P.h.n = plan.n;
   P.h.m = sw.m;
   P.h.L = sw.L;
-  const int rq = rq_override > 0 ? rq_override : reg_qubits_for(sw.m);
+  const int rq = rq_override > 0 ? rq_override : plan.lane ? kMaxRegQ : reg_qubits_for(sw.m);
   P.h.rq = rq;
+  P.h.lane = plan.lane ? 1 : 0;
   P.h.nops = (int)sw.ops.size();
   int loc[64];
   for (int q = 0; q < 64; q++) loc[q] = -1;
@@ -78,7 +79,7 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
     P.h.tq[i] = (int8_t)sw.tq[i];
     loc[sw.tq[i]] = i;
   }
-  const bool reg_ok = sw.m >= rq && sw.m - rq <= 8;
+  const bool reg_ok = sw.m >= rq && (plan.lane || sw.m - rq <= 8);
   struct Tmp {
     DevOp d;
     std::vector<cplx> m;
@@ -497,6 +498,40 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
       flush();
       return fold_diag(t);
     };
+    // Carries the table across a bit flip or a swap: the op only permutes the
+    // register combinations (where its controls hold), so T before it is the
+    // permuted T after it.  Controls on thread bits or outside the tile become
+    // selectors.  (A CNOT ladder between rotations would otherwise cost a
+    // table per CNOT: 143 tables for the 47 phases of a 12-qubit ansatz of ten
+    // layers, 77 with this; a table is four FP64 instructions an amplitude.)
+    auto carry = [&](const Tmp& t) {
+      const DevOp& d = t.d;
+      const bool flip = d.kind == OPK_ANTIDIAG && (d.pad & OPF_FLIP);
+      if (!plan.carry_flips || !(flip || d.kind == OPK_SWAP)) return false;
+      std::vector<int> codes;
+      if (!need_codes(d, codes)) return false;
+      for (int c : codes) selector(c);
+      std::vector<cplx> to = tab;
+      for (int v = 0; v < nvar(); v++) {
+        bool on = true;
+        for (int c : codes) {
+          const bool want = c < 64 ? (d.tval >> c) & 1u : (d.xval >> (c - 64)) & 1ull;
+          on = on && (((v >> selector(c)) & 1) != 0) == want;
+        }
+        if (!on) continue;
+        for (int j = 0; j < NT; j++) {
+          if (((uint32_t)j & d.rmask) != d.rval) continue;
+          int k = j ^ (1 << d.rs[0]);
+          if (!flip) {
+            const int x = ((j >> d.rs[0]) ^ (j >> d.rs[1])) & 1;
+            k = j ^ (x << d.rs[0]) ^ (x << d.rs[1]);
+          }
+          to[v * NT + k] = tab[v * NT + j];
+        }
+      }
+      tab = std::move(to);
+      return true;
+    };
     for (int o = first; o < first + nops;) {
       const Tmp& t = ts[o];
       const DevOp& d = t.d;
@@ -586,7 +621,7 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
         uint32_t tg = 0;
         for (int i = 0; i < d.k; i++)
           if (d.rs[i] != 0xFF) tg |= 1u << d.rs[i];
-        if (tab_dep(tg)) flush();
+        if (tab_dep(tg) && !carry(t)) flush();
       }
       fin.push_back(t);
       o++;
@@ -962,7 +997,8 @@ extern "C" sv_status sv_emulate_apply(int n_qubits, sv_dtype dtype, const sv_gat
     sv_exec_opts o;
     std::memset(&o, 0, sizeof(o));
     if (opts) o = *opts;
-    const Plan plan = make_plan(n_qubits, dtype, gates, n_gates, param_values, n_param_values, o);
+    const Plan plan = make_plan(n_qubits, dtype, gates, n_gates, param_values, n_param_values, o, 0,
+                                lane_sizes(n_qubits, o));
     zc* st = reinterpret_cast<zc*>(state);
     if (dtype == SV_C64) {
       std::unique_ptr<SweepProgram<float>> P(new SweepProgram<float>());

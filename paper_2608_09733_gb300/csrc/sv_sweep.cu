@@ -839,6 +839,10 @@ cudaError_t launch_sweep(Cx<R>* state, const SweepProgram<R>& prog, cudaStream_t
   // take the TMA pass, with the program's compiled kernel when it has one
   bool used = false, used_jit = false;
   if (kernel) *kernel = "sweep";
+  if (prog.h.lane) {
+    if (kernel) *kernel = "sweep_lane";
+    return launch_lane_pass<R>(state, prog, stream);
+  }
   if constexpr (sizeof(R) == 4) {
     if (prog.h.rq == 5) {
       cudaError_t e = launch_sweep_tma<R, 5>(state, prog, stream, used, jit, used_jit);
