@@ -12,17 +12,21 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <list>
 #include <map>
 #include <memory>
 #include <mutex>
+#include <thread>
 #include <tuple>
 
 #include "sv_hostcopy.h"
 #include "sv_internal.h"
+#include "sv_stage.cuh"
 
 namespace sv {
 namespace {
@@ -622,43 +626,104 @@ sv_status sv_profile_read(sv_profile_entry* out, int max_entries, int* n_out, in
 
 namespace sv {
 namespace {
+
+// f(i) for i in 0..n-1 on up to one host thread per core (requests are
+// independent; planning one takes about 0.2 ms).  The error of the lowest
+// index is raised, as a loop would; a thread that cannot be started is done
+// without.
+template <typename F>
+void for_each_request(int n, F&& f) {
+  std::atomic<int> next{0};
+  std::mutex mu;
+  int failed = n;
+  std::exception_ptr error;
+  auto work = [&] {
+    for (int i; (i = next.fetch_add(1)) < n;) {
+      try {
+        f(i);
+      } catch (...) {
+        std::lock_guard<std::mutex> lk(mu);
+        if (i < failed) {
+          failed = i;
+          error = std::current_exception();
+        }
+      }
+    }
+  };
+  const unsigned cores = std::max(1u, std::thread::hardware_concurrency());
+  const int extra = std::min((int)std::min(cores, 32u), n / 4) - 1;  // below four requests a thread costs more than it saves
+  std::vector<std::thread> threads;
+  try {
+    for (int t = 0; t < extra; t++) threads.emplace_back(work);
+  } catch (...) {
+  }
+  work();
+  for (std::thread& t : threads) t.join();
+  if (error) std::rethrow_exception(error);
+}
+
 template <typename R>
 void run_batch_small(int nreq, sv_dtype dtype, const int* nq, const sv_gate* const* gates, const size_t* ng,
                      double* out, int out_on_device, cudaStream_t stream) {
-  std::vector<Plan> plans;
-  plans.reserve(nreq);
-  size_t nprog = 0;
-  int max_n = 1;
   sv_exec_opts o;
   std::memset(&o, 0, sizeof(o));
+  // Each request is planned and its programs built by one thread, which frees
+  // the plan again: a program is kept cut after its last coefficient (about 14
+  // of 32 KB).
+  struct Request {
+    std::vector<char> bytes;       // its programs, back to back
+    std::vector<uint32_t> offset;  // of each program in bytes
+  };
+  std::vector<Request> req(nreq);
+  for_each_request(nreq, [&](int b) {
+    const Plan plan = make_plan(nq[b], dtype, gates[b], ng[b], nullptr, 0, o, nq[b]);
+    std::unique_ptr<SweepProgram<R>> prog(new SweepProgram<R>());
+    for (const Sweep& sw : plan.sweeps) {
+      build_program<R>(plan, sw, *prog, kRegQ);
+      const char* p = reinterpret_cast<const char*>(prog.get());
+      req[b].offset.push_back((uint32_t)req[b].bytes.size());
+      req[b].bytes.insert(req[b].bytes.end(), p, p + staged_bytes<R>(prog->h.ncoef));
+    }
+  });
+  // Staging: the index (first program of each request, qubits of each request,
+  // byte offset of each program), then the programs.
+  size_t nprog = 0, prog_bytes = 0;
+  int max_n = 1;
+  std::vector<size_t> start(nreq);  // of each request's programs, after the index
   for (int b = 0; b < nreq; b++) {
-    plans.push_back(make_plan(nq[b], dtype, gates[b], ng[b], nullptr, 0, o, nq[b]));
-    nprog += plans.back().sweeps.size();
+    start[b] = prog_bytes;
+    nprog += req[b].offset.size();
+    prog_bytes += req[b].bytes.size();
     max_n = std::max(max_n, nq[b]);
   }
-  const size_t prog_bytes = sizeof(SweepProgram<R>) * nprog;
-  const size_t idx_bytes = sizeof(int) * (2 * (size_t)nreq + 1);
-  const size_t total = prog_bytes + idx_bytes;
-  Pinned& pb = pinned_buffer(stream, "small_batch_staging", total);
-  SweepProgram<R>* hp = reinterpret_cast<SweepProgram<R>*>(pb.p);
-  int* hfirst = reinterpret_cast<int*>(reinterpret_cast<char*>(pb.p) + prog_bytes);
+  const size_t int_bytes = (sizeof(int) * (2 * (size_t)nreq + 1) + 15) / 16 * 16;
+  const size_t idx_bytes = int_bytes + sizeof(uint64_t) * ((nprog + 1) / 2 * 2);
+  const size_t total = idx_bytes + prog_bytes;
+  const size_t most = idx_bytes + sizeof(SweepProgram<R>) * nprog;  // grown by program count, not by content
+  Pinned& pb = pinned_buffer(stream, "small_batch_staging", most);
+  char* base = reinterpret_cast<char*>(pb.p);
+  int* hfirst = reinterpret_cast<int*>(base);
   int* hnq = hfirst + nreq + 1;
-  size_t k = 0;
+  uint64_t* hoff = reinterpret_cast<uint64_t*>(base + int_bytes);
+  hfirst[0] = 0;
   for (int b = 0; b < nreq; b++) {
-    hfirst[b] = (int)k;
+    hfirst[b + 1] = hfirst[b] + (int)req[b].offset.size();
     hnq[b] = nq[b];
-    for (const Sweep& sw : plans[b].sweeps) build_program<R>(plans[b], sw, hp[k++], kRegQ);
   }
-  hfirst[nreq] = (int)k;
-  char* dbuf = (char*)scratch_buffer(stream, "small_batch_programs", total);
+  for_each_request(nreq, [&](int b) {
+    for (size_t i = 0; i < req[b].offset.size(); i++) hoff[hfirst[b] + i] = idx_bytes + start[b] + req[b].offset[i];
+    if (!req[b].bytes.empty()) std::memcpy(base + idx_bytes + start[b], req[b].bytes.data(), req[b].bytes.size());
+    req[b] = Request();
+  });
+  char* dbuf = (char*)scratch_buffer(stream, "small_batch_programs", most);
   cuda_check(cudaMemcpyAsync(dbuf, pb.p, total, cudaMemcpyHostToDevice, stream), "program upload");
   cuda_check(cudaEventRecord(pb.ready, stream), "cudaEventRecord");
-  const SweepProgram<R>* dp = reinterpret_cast<const SweepProgram<R>*>(dbuf);
-  const int* dfirst = reinterpret_cast<const int*>(dbuf + prog_bytes);
+  const int* dfirst = reinterpret_cast<const int*>(dbuf);
   const int* dnq = dfirst + nreq + 1;
+  const uint64_t* doff = reinterpret_cast<const uint64_t*>(dbuf + int_bytes);
   double* dout = out_on_device ? out : (double*)scratch_buffer(stream, "small_batch_out", sizeof(double) * nreq);
   Prof pr(stream, "small_batch", 0.0);
-  cuda_check(launch_small_batch<R>(dp, dfirst, dnq, nreq, max_n, dout, stream), "small batch launch");
+  cuda_check(launch_small_batch<R>(dbuf, doff, dfirst, dnq, nreq, max_n, dout, stream), "small batch launch");
   pr.done();
   if (!out_on_device) {
     cuda_check(cudaMemcpyAsync(out, dout, sizeof(double) * nreq, cudaMemcpyDeviceToHost, stream), "result copy");

@@ -148,9 +148,10 @@ bool lane_pass_available();
 template <typename R>
 cudaError_t launch_init_basis(Cx<R>* state, int n, uint64_t index, cudaStream_t stream);
 // One CTA per small request (whole state in shared memory): request b runs
-// programs first_prog[b] .. first_prog[b+1]-1 and writes sum_q <Z_q> to out[b].
+// programs first_prog[b] .. first_prog[b+1]-1 (program p at buf + offset[p],
+// device memory) and writes sum_q <Z_q> to out[b].
 template <typename R>
-cudaError_t launch_small_batch(const SweepProgram<R>* progs, const int* first_prog, const int* nq, int n_requests,
+cudaError_t launch_small_batch(const char* buf, const uint64_t* offset, const int* first_prog, const int* nq, int n_requests,
                                int max_n, double* out, cudaStream_t stream);
 
 // Persistent packed small states (serving sessions, sv_serve.cpp).  The
