@@ -387,7 +387,7 @@ void segment_programs(const AdjTemplate& T, size_t g0, size_t g1, bool reverse, 
       ops.push_back(T.ag[i].op);
     }
   }
-  std::vector<Sweep> sws = schedule_sweeps(n, ops, tile_q, low_q, BatchProgram<R>::kPool / 2, 64);
+  std::vector<Sweep> sws = schedule_sweeps(n, ops, tile_q, low_q, BatchProgram<R>::kPool / 2, 64, false);
   for (const Sweep& sw : sws) {
     fill_program<R>(T.ag, order, sw, n, batch, T.npg, reverse, prog);
     each(prog);

@@ -44,9 +44,10 @@ struct Plan {
   std::vector<int> block_starts;  // first gate of each op (fusion blocks) + n_gates
   std::vector<Sweep> sweeps;
   bool lane = false;        // passes of the cluster kernel (sv_lane.cu): tiles of up to 2^14 amplitudes
-  // phase tables are carried across bit flips and swaps (permuted) instead of
-  // applied before them; not for the packed and session programs, whose
-  // rounding stays as it is
+  // programs whose ops may be reordered over their phases and whose phase
+  // tables are carried across bit flips and swaps (permuted) instead of applied
+  // before them; not the packed and session programs, whose rounding stays as
+  // it is
   bool carry_flips = false;
 };
 
@@ -104,7 +105,7 @@ std::vector<LOp> fuse_greedy(int n, const sv_gate* gates, size_t n_gates, const 
                              std::vector<int>* block_starts, bool dense_always);
 void classify(LOp& op);
 std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_q, int low_q, int coef_pool,
-                                   int ops_per_pass);
+                                   int ops_per_pass, bool commute);
 Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, const double* param_values,
                size_t n_param_values, const sv_exec_opts& opts, int tile_q_override = 0, bool lane = false);
 // Whether a state of this size with these options takes the cluster pass.
@@ -124,6 +125,21 @@ struct RotSplit {
   double C = 1.0, S = 0.0;
 };
 bool rot_split(const cplx* U, double tol, RotSplit& r);
+
+// An op as the phases see it: the qubits it acts on other than diagonally and
+// diagonally (controls, diagonals), the local positions it needs as register
+// slots, and whether it runs in shared memory (a phase of its own).
+struct PhaseOp {
+  uint64_t moves, holds;
+  uint32_t need;
+  bool smem;
+};
+PhaseOp phase_op(const LOp& op, uint32_t need, bool smem);
+// The ops of a pass ordered by phases of rq register slots: a phase takes, in
+// order, every op whose slots still fit and that commutes with each op passed
+// over before it.  *phases: the phases of that order; *runs: of the given
+// order, a phase ending at the first op that does not fit.
+std::vector<int> order_by_phase(const std::vector<PhaseOp>& ops, int rq, int* phases, int* runs);
 
 template <typename R>
 void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override = 0);

@@ -23,12 +23,12 @@
 // memory and each op's descriptor is loaded one op ahead.
 //
 // Measured (us a circuit, one CTA a tile -> here): 12 qubits complex128, ten
-// RY/RZ/CNOT layers 690 -> 183; 20 layers of U3 and CZ 700 -> 236; 300 random
-// one- and two-qubit matrices 1640 -> 314; complex64, U3 and CNOT ladder of
-// depth 22, 8 qubits 156 -> 115, 12 qubits 261 -> 241, 14 qubits 428 -> 383.
-// A pass of the 12-qubit ansatz runs 8800 instructions a warp at a latency of
-// 11 cycles each (shared-memory round trips of shuffles and operands), its
-// FP64 pipe busy a third of the time: the serial chain still bounds it.
+// RY/RZ/CNOT layers 690 -> 162; 14 qubits, 20 layers of U3 and CZ 811 -> 542;
+// complex64, U3 and CNOT ladder of depth 22 on 15 qubits 465 -> 303; 200 one-
+// and 100 two-qubit random matrices on 13 qubits 476 -> 77 (joined matrices,
+// two passes).  A pass of the 12-qubit ansatz waits about 11 cycles an
+// instruction (shared-memory round trips of shuffles and operands), its FP64
+// pipe busy a third of the time: the serial chain still bounds it.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -115,7 +115,9 @@ struct OpWords {
   __device__ __forceinline__ uint32_t k() const { return (a.x >> 8) & 255u; }
   __device__ __forceinline__ uint32_t pos(int i) const { return (a.x >> (16 + 8 * i)) & 255u; }  // i < 2
   __device__ __forceinline__ uint32_t gq(int i) const { return (a.w >> (8 * i)) & 255u; }         // i < 4
-  __device__ __forceinline__ uint32_t rs(int i) const { return (b.x >> (8 + 8 * i)) & 255u; }     // i < 3
+  __device__ __forceinline__ uint32_t rs(int i) const { return (i < 3 ? b.x >> (8 + 8 * i) : b.y) & 255u; }  // i < 4
+  __device__ __forceinline__ uint32_t lmask() const { return b.z; }
+  __device__ __forceinline__ uint32_t lval() const { return b.w; }
   __device__ __forceinline__ uint32_t tmask() const { return c.x; }
   __device__ __forceinline__ uint32_t tval() const { return c.y; }
   __device__ __forceinline__ uint64_t xmask() const { return c.z | ((uint64_t)c.w << 32); }
@@ -124,7 +126,8 @@ struct OpWords {
   __device__ __forceinline__ uint32_t code() const { return d.w; }
 };
 static_assert(offsetof(DevOp, k) == 1 && offsetof(DevOp, pos) == 2 && offsetof(DevOp, gq) == 12 &&
-                  offsetof(DevOp, rs) == 17 && offsetof(DevOp, tmask) == 32 && offsetof(DevOp, tval) == 36 &&
+                  offsetof(DevOp, rs) == 17 && offsetof(DevOp, lmask) == 24 && offsetof(DevOp, lval) == 28 &&
+                  offsetof(DevOp, tmask) == 32 && offsetof(DevOp, tval) == 36 &&
                   offsetof(DevOp, xmask) == 40 && offsetof(DevOp, xval) == 48 && offsetof(DevOp, coef) == 56 &&
                   offsetof(DevOp, pad) == 60,
               "OpWords reads DevOp by word");
@@ -262,6 +265,27 @@ __device__ __forceinline__ void lane_op(Cx<R> (&v)[A], const OpWords& op, const 
           if (lane_on) v[a] = p;
         }
       }
+      break;
+    }
+    case OPK_PERM: {
+      uint32_t from = op.lval();
+#pragma unroll
+      for (int q = 0; q < 5; q++) from ^= (lane >> q) & 1u ? (op.lmask() >> (5 * q)) & 31u : 0u;
+      uint32_t src[A];
+#pragma unroll
+      for (int a = 0; a < A; a++) src[a] = from;
+      const uint32_t k = op.k();
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        if (i >= k) continue;
+        const uint32_t c = op.gq(i), v_i = op.rs(i);
+        const uint32_t x = (uint32_t)(base >> (c & 63u));
+#pragma unroll
+        for (int a = 0; a < A; a++) src[a] ^= (c < 64 ? tb[a] >> (c & 31u) : x) & 1u ? v_i : 0u;
+      }
+#pragma unroll
+      for (int a = 0; a < A; a++)
+        v[a] = Cx<R>{__shfl_sync(0xffffffffu, v[a].re, src[a]), __shfl_sync(0xffffffffu, v[a].im, src[a])};
       break;
     }
     case OPK_SWAP: {

@@ -410,8 +410,19 @@ static int coef_count(const LOp& op) {
   }
 }
 
+PhaseOp phase_op(const LOp& op, uint32_t need, bool smem) {
+  uint64_t t = 0;
+  if (op.kind != OPK_DIAG)
+    for (int i = 0; i < op.k; i++) t |= 1ull << op.q[i];
+  return {t, op.touch & ~t, need, smem};
+}
+
+// With `commute` an op may go before ops passed over when on every qubit it
+// shares with them both act diagonally (controls and diagonals commute), not
+// only when it shares none: CZ layers then hold up fewer ops (20 layers of U3
+// and CZ on 30 qubits: 35 passes against 38, on 24 qubits 25 against 28).
 std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_q, int low_q, int coef_pool,
-                                   int ops_per_pass) {
+                                   int ops_per_pass, bool commute) {
   const int max_ops = ops_per_pass > 0 ? std::min(ops_per_pass, kMaxOps) : kMaxOps;
   std::vector<Sweep> out;
   const int m_max = std::min(n, tile_q);
@@ -422,27 +433,26 @@ std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_
   while (ndone < ops.size()) {
     Sweep sw;
     uint64_t S = (1ull << L0) - 1ull;
-    uint64_t blocked = 0;
+    uint64_t moved = 0, held = 0;  // qubits the ops passed over act on: other than diagonally, diagonally
     int coef = 0;
     for (size_t i = first; i < ops.size(); i++) {
       if (done[i]) continue;
       const LOp& op = ops[i];
-      if (op.touch & blocked) {
-        blocked |= op.touch;
-        if ((blocked & all) == all) break;
-        continue;
-      }
+      PhaseOp p = phase_op(op, 0, false);
+      if (!commute) p = {op.touch, 0, 0, false};
+      const bool blocked = (p.moves & (moved | held)) || (p.holds & moved);
       uint64_t S2 = S | op.need;
       int c = coef_count(op);
-      if (popc(S2) <= m_max && (int)sw.ops.size() < max_ops && coef + c <= coef_pool) {
+      if (!blocked && popc(S2) <= m_max && (int)sw.ops.size() < max_ops && coef + c <= coef_pool) {
         S = S2;
         coef += c;
         sw.ops.push_back((int)i);
         done[i] = 1;
         ndone++;
       } else {
-        blocked |= op.touch;
-        if ((blocked & all) == all) break;
+        moved |= p.moves;
+        held |= p.holds;
+        if ((moved & all) == all) break;
       }
     }
     if (sw.ops.empty()) fail(SV_ERR_INVALID, "scheduler could not place an operation");
@@ -457,6 +467,46 @@ std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_
     while (first < ops.size() && done[first]) first++;
   }
   return out;
+}
+
+std::vector<int> order_by_phase(const std::vector<PhaseOp>& ops, int rq, int* phases, int* runs) {
+  const int n = (int)ops.size();
+  std::vector<char> done(n, 0);
+  std::vector<int> seq;
+  seq.reserve(n);
+  *phases = *runs = 0;
+  for (int first = 0; (int)seq.size() < n;) {
+    (*phases)++;
+    while (done[first]) first++;
+    uint64_t moved = 0, held = 0;  // by the ops passed over
+    uint32_t need = 0;
+    bool alone = false;
+    for (int o = first; o < n && !alone; o++) {
+      if (done[o]) continue;
+      const PhaseOp& p = ops[o];
+      // of two ops, the later may go first when on every qubit they share
+      // both act diagonally
+      const bool blocked = (p.moves & (moved | held)) || (p.holds & moved);
+      if (!blocked && (p.smem ? o == first : popc(need | p.need) <= rq)) {
+        done[o] = 1;
+        seq.push_back(o);
+        need |= p.need;
+        alone = p.smem;
+        continue;
+      }
+      moved |= p.moves;
+      held |= p.holds;
+    }
+  }
+  uint32_t need = 0;
+  bool open = false;
+  for (const PhaseOp& p : ops) {
+    const bool joins = open && !p.smem && popc(need | p.need) <= rq;
+    if (!joins) (*runs)++;
+    need = p.smem ? 0u : joins ? need | p.need : p.need;
+    open = !p.smem;
+  }
+  return seq;
 }
 
 // An uncontrolled complex one-qubit op g diag(1, ephi) R diag(1, elam)
@@ -673,9 +723,10 @@ static void defer_diagonals(const std::vector<LOp>& ops, std::vector<Sweep>& sw,
 // States of up to four cluster tiles (2^14 amplitudes each) take the cluster
 // pass: a tile spread over a cluster's SMs, an amplitude a lane.  At 17 qubits
 // the eight clusters no longer fit beside each other and the one-CTA tiles,
-// 16 of them by then, are faster (complex64, U3 + CNOT ladder of depth 22:
-// 15 qubits 430 against 461 us, 16 qubits 472 against 465 but 287 against 456
-// on random two-qubit matrices, 17 qubits 840 against 552).  Below five
+// 16 of them by then, are faster (measured before phases were ordered;
+// complex64, U3 + CNOT ladder of depth 22: 15 qubits 430 against 461 us, 16
+// qubits 472 against 465 but 287 against 456 on random two-qubit matrices, 17
+// qubits 840 against 552).  Below five
 // qubits there is no warp to fill.  An explicit tile width or cap of
 // operations per pass keeps its own kernel.
 bool lane_sizes(int n, const sv_exec_opts& opts) {
@@ -736,16 +787,25 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
                      : opts.tile_qubits > 0 ? std::min(opts.tile_qubits, n)
                                             : tile_qubits_for(dtype, n);
   const int max_ops = opts.ops_per_pass > 0 ? std::min(opts.ops_per_pass, kMaxOps) : kMaxOps;
-  p.sweeps = schedule_sweeps(n, p.ops, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass);
+  // The packed and session programs keep their order.  So do complex128 passes
+  // of many tiles: the FP64 pipe bounds them, and an order with fewer passes
+  // has more tables (20 layers of U3 and CZ on 24 qubits: 28 passes 48.3 ms,
+  // 29 passes 46.3).
+  const bool commute = tile_q_override == 0 && (dtype == SV_C64 || lane);
+  p.sweeps = schedule_sweeps(n, p.ops, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass, commute);
   if (opts.ops_per_pass != 1) {
     defer_diagonals(p.ops, p.sweeps, max_ops, pool);
     // The split form has more ops, which can cut the greedy passes short and
-    // leave more of them: keep it only when it needs no more passes.
+    // leave more of them: keep it only when it needs no more passes, or at most
+    // one in twenty more.  Whole gates close with a table of their own in each
+    // phase: 20 layers of U3 and CZ on 28 qubits take 31.8 ms with 32 passes
+    // and 252 tables, 28.7 ms with 33 passes and 162.
     std::vector<LOp> ops2 = p.ops;
     split_one_qubit(ops2, dtype == SV_C64 ? 1e-9 : 1e-13);
     drop_identities(ops2);
-    std::vector<Sweep> sw2 = schedule_sweeps(n, ops2, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass);
-    if (sw2.size() <= p.sweeps.size()) {
+    std::vector<Sweep> sw2 = schedule_sweeps(n, ops2, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass, commute);
+    const size_t more = commute ? p.sweeps.size() / 20 : 0;
+    if (sw2.size() <= p.sweeps.size() + more) {
       defer_diagonals(ops2, sw2, max_ops, pool);
       p.ops = std::move(ops2);
       p.sweeps = std::move(sw2);

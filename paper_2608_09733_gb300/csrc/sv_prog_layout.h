@@ -44,6 +44,10 @@ enum OpKind : uint8_t {
   OPK_PHASE = 8,    // register phase only: amplitude j of the thread's 2^RQ is multiplied by
                     // coef[var * table_stride(RQ) + j]; var collects k selector bits, selector i being bit
                     // gq[i] of the thread's local bits (gq[i] < 64) or global bit gq[i] - 64 of the tile
+  OPK_PERM = 9,     // register phase of a cluster pass only: a run of bit flips and swaps as one map of the
+                    // register index, amplitude j taken from A j ^ c ^ (v_i for each set bit i): lmask holds
+                    // A's columns (five bits each), lval c, and entry i < k the bit gq[i] (a local bit of the
+                    // thread, or 64 + a global bit of the tile) and its v_i = rs[i]
 };
 
 // DevOp.pad flag bits

@@ -63,8 +63,10 @@ bool rot_split(const cplx* U, double tol, RotSplit& r) {
 // positions and control masks; consecutive ops whose moving qubits fit four
 // register slots form one register phase; dense k >= 3 blocks and wide
 // diagonals get a shared-memory phase of their own.
+// order: 0 keeps the pass's op order, 1 orders by phases where the rule below
+// says so, 2 always.
 template <typename R>
-void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override) {
+void build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override, int order_by) {
   std::memset(&P.h, 0, sizeof(P.h));
   P.h.n = plan.n;
   P.h.m = sw.m;
@@ -277,6 +279,41 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
       }
     }
   };
+  // The order of the ops over the phases.  A phase takes, in order, every op
+  // whose moving qubits still fit its register slots and that commutes with
+  // each op passed over before it, not only the run of ops up to the first
+  // that does not fit: of two ops, the later may go first when on every qubit
+  // they share both act diagonally (as a control or a diagonal).  That takes
+  // about 40 % fewer phases and up to 30 % more tables (20 layers of U3 and CZ
+  // on 24 qubits: 63 phases and 178 tables; 22 layers of U3 and CNOT ladder on
+  // 17: 78 phases and 199 tables against 131 and 219).  Complex64 states of 25
+  // qubits and more stream from HBM in compiled passes, where a table
+  // costs as much as a phase: they take this order only where it saves three
+  // phases of a pass (a 30-qubit pass of 7 phases 7.85 ms, of 4 phases and
+  // three more tables 5.92; one of 4 phases 4.35 ms, of 3 phases and two more
+  // tables 4.80).
+  if (plan.carry_flips && order_by) {
+    const int nt = (int)ts.size();
+    std::vector<PhaseOp> pops(nt);
+    for (int o = 0; o < nt; o++) {
+      const LOp& op = plan.ops[sw.ops[order[o]]];
+      pops[o] = phase_op(op, ts[o].need, ts[o].smem);
+    }
+    int phases = 0, runs = 0;
+    const std::vector<int> seq = order_by_phase(pops, rq, &phases, &runs);
+    const bool streams = sizeof(R) == 4 && plan.n >= 25;
+    if (order_by == 2 || runs - phases >= (streams ? 3 : 1)) {
+      std::vector<Tmp> ts2;
+      std::vector<int> at2;
+      ts2.reserve(nt);
+      for (int o : seq) {
+        ts2.push_back(std::move(ts[o]));
+        at2.push_back(ts_attach[o]);
+      }
+      ts = std::move(ts2);
+      ts_attach = std::move(at2);
+    }
+  }
   // Greedy register phases.  Diagonals attached forward wait for their op and
   // open its phase with it; the others join the phase in progress.
   int cur_first = -1, cur_n = 0, pend = 0;
@@ -628,6 +665,58 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
     }
     flush();
   };
+  // Runs of X, CNOT (either control state) and SWAP in fin[at ..] as one map of
+  // the register index each (OPK_PERM); a run ends where its map would depend
+  // on more than four bits outside the register.
+  auto merge_flips = [&](size_t at) {
+    std::vector<Tmp> list(std::make_move_iterator(fin.begin() + at), std::make_move_iterator(fin.end()));
+    fin.resize(at);
+    for (size_t i = 0; i < list.size();) {
+      uint32_t col[kMaxRegQ], c = 0;
+      for (int q = 0; q < kMaxRegQ; q++) col[q] = 1u << q;
+      std::vector<std::pair<int, uint32_t>> bits;  // code, v
+      size_t j = i;
+      for (; j < list.size(); j++) {
+        const DevOp& d = list[j].d;
+        const int controls = __builtin_popcount(d.rmask) + __builtin_popcount(d.tmask) + __builtin_popcountll(d.xmask);
+        if (d.kind == OPK_SWAP && controls == 0) {
+          std::swap(col[d.rs[0]], col[d.rs[1]]);
+          continue;
+        }
+        if (!(d.kind == OPK_ANTIDIAG && (d.pad & OPF_FLIP) && controls <= 1)) break;
+        const uint32_t v = col[d.rs[0]];
+        bool when_set = true;
+        if (d.rmask) {
+          when_set = d.rval != 0;
+          col[__builtin_ctz(d.rmask)] ^= v;
+        } else if (controls) {
+          const int code = d.tmask ? __builtin_ctz(d.tmask) : 64 + __builtin_ctzll(d.xmask);
+          when_set = d.tmask ? d.tval != 0 : d.xval != 0;
+          size_t b = 0;
+          while (b < bits.size() && bits[b].first != code) b++;
+          if (b == 4) break;
+          if (b == bits.size()) bits.emplace_back(code, 0u);
+          bits[b].second ^= v;
+        }
+        if (!controls || !when_set) c ^= v;
+      }
+      if (j - i < 2) {  // nothing to merge
+        fin.push_back(std::move(list[i]));
+        i++;
+        continue;
+      }
+      Tmp t = blank(OPK_PERM);
+      for (int q = 0; q < kMaxRegQ; q++) t.d.lmask |= col[q] << (5 * q);
+      t.d.lval = c;
+      t.d.k = (uint8_t)bits.size();
+      for (size_t b = 0; b < bits.size(); b++) {
+        t.d.gq[b] = (uint8_t)bits[b].first;
+        t.d.rs[b] = (uint8_t)bits[b].second;
+      }
+      fin.push_back(std::move(t));
+      i = j;
+    }
+  };
   // Builds the whole list; false if it does not fit the program (the table
   // form can need more ops and coefficients than the plain one).
   auto make_fin = [&](bool rot, int max_sel) {
@@ -644,10 +733,11 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
           emit_phase_rot(first, nops, max_sel);
         else
           emit_phase_plain(first, nops);
+        if (plan.lane) merge_flips(nf);
         for (int i = nf; i < (int)fin.size(); i++) {
           DevOp& d = fin[i].d;
           d.pad &= OPF_FLIP;
-          if (d.kind != OPK_KRON && d.kind != OPK_KROT && d.kind != OPK_PHASE) {
+          if (d.kind != OPK_KRON && d.kind != OPK_KROT && d.kind != OPK_PHASE && d.kind != OPK_PERM) {
             if (d.tmask) d.pad |= OPF_TCOND;
             if (d.xmask) d.pad |= OPF_XCOND;
           }
@@ -715,6 +805,28 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
     }
     std::fprintf(stderr, "\n");
   }
+}
+
+// Complex128 passes of many tiles are bound by the FP64 pipe: a table is four
+// instructions an amplitude, a phase none, so both orders are built and the
+// one with fewer tables is kept (by less than two phases a table).
+template <typename R>
+void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override) {
+  if (!(sizeof(R) == 8 && plan.carry_flips && !plan.lane)) {
+    build_program_ordered<R>(plan, sw, P, rq_override, 1);
+    return;
+  }
+  auto cost = [](const SweepProgram<R>& p) {
+    int tables = 0;
+    for (int i = 0; i < p.h.nphases; i++)
+      if (p.ph[i].kind == PH_REG)
+        for (int o = p.ph[i].first; o < p.ph[i].first + p.ph[i].nops; o++) tables += (p.ops[o].pad & 15u) == OPK_PHASE;
+    return 2 * tables + p.h.nphases;
+  };
+  build_program_ordered<R>(plan, sw, P, rq_override, 0);
+  std::unique_ptr<SweepProgram<R>> other(new SweepProgram<R>());
+  build_program_ordered<R>(plan, sw, *other, rq_override, 2);
+  if (cost(*other) < cost(P)) std::memcpy(&P, other.get(), sizeof(P));
 }
 
 template void build_program<float>(const Plan&, const Sweep&, SweepProgram<float>&, int);
@@ -837,6 +949,21 @@ void emulate_reg_op(const SweepProgram<R>& P, const DevOp& op, uint32_t code, in
         }
       });
       break;
+    case OPK_PERM: {
+      uint32_t c = op.lval;
+      for (int i = 0; i < op.k; i++) {
+        const uint32_t bit = op.gq[i] < 64 ? (tb >> op.gq[i]) & 1u : (uint32_t)(base >> (op.gq[i] - 64)) & 1u;
+        if (bit) c ^= op.rs[i];
+      }
+      const std::vector<zc> in = v;
+      for (int j = 0; j < NR; j++) {
+        uint32_t from = c;
+        for (int q = 0; q < rq; q++)
+          if ((j >> q) & 1) from ^= (op.lmask >> (5 * q)) & 31u;
+        v[j] = in[from];
+      }
+      break;
+    }
     case OPK_SWAP: {
       const int A = op.rs[0], B = op.rs[1];
       for (int j = 0; j < NR; j++) {
