@@ -28,7 +28,7 @@ namespace {
 
 
 template <typename R, bool REV>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(256, batch_resident(sizeof(R), REV))
     k_batch_sweep(Cx<R>* __restrict__ psi, Cx<R>* __restrict__ lam, const Cx<R>* __restrict__ table,
                   double* __restrict__ gscratch, const __grid_constant__ BatchProgram<R> P) {
   batch_sweep_body<R, REV>(psi, lam, table, gscratch, P, BatchInterp<R, REV>{P});
@@ -259,12 +259,25 @@ __global__ void k_sum_rows(const double* __restrict__ in, int rows, int cols, do
 
 }  // namespace
 
-int batch_grid_x(int n, int m, int batch) {
-  // about four resident CTAs per SM over the whole batch, at most one per tile
-  int want = (device_sm_count() * 4 + batch - 1) / batch;
-  uint64_t tiles = 1ull << (n - m);
-  if ((uint64_t)want > tiles) want = (int)tiles;
-  return want < 1 ? 1 : want;
+// CTAs per state: the count that finishes first when the CTAs of all states
+// run in waves of `per_sm` an SM, a CTA costing its tiles and about half a tile
+// for its setup.  (Four CTAs an SM over the batch, rounded up per state, gave
+// 64 states of 256 tiles ten CTAs each: 640 CTAs on 304 places, a third wave of
+// 32.  19 CTAs are four full waves of 14 tiles: 56 tile times against 78.)
+int batch_grid_x(int n, int m, int batch, int per_sm) {
+  const uint64_t tiles = 1ull << (n - m), places = (uint64_t)device_sm_count() * per_sm;
+  const uint64_t most = std::min<uint64_t>(tiles, std::max<uint64_t>(1, 8 * places / batch));
+  uint64_t best = 1;
+  double best_cost = 0.0;
+  for (uint64_t g = 1; g <= most; g++) {
+    const double waves = (double)((g * batch + places - 1) / places);
+    const double cost = waves * ((double)((tiles + g - 1) / g) + 0.5);
+    if (g == 1 || cost < best_cost) {
+      best = g;
+      best_cost = cost;
+    }
+  }
+  return (int)best;
 }
 
 template <typename R>

@@ -17,7 +17,7 @@ template <typename R>
 cudaError_t launch_batch_sweep(Cx<R>* psi, Cx<R>* lam, const Cx<R>* table, double* gscratch, int grid_x,
                                const BatchProgram<R>& prog, bool reverse, cudaStream_t stream,
                                const JitKernel* jit = nullptr);
-int batch_grid_x(int n, int m, int batch);
+int batch_grid_x(int n, int m, int batch, int per_sm);
 template <typename R>
 cudaError_t launch_batch_init(Cx<R>* psi, int n, int batch, cudaStream_t stream);
 // lam (=|+=) sum_j c_j P_j psi over the terms sharing one x mask

@@ -200,6 +200,66 @@ AdjTemplate lower_template(const sv_gate* gates, size_t ng) {
   return T;
 }
 
+// The ops of one register phase with its uncontrolled one-qubit diagonals
+// (without a gradient, or with the Z generator) gathered into groups.  Such an
+// op may move anywhere between the ops that target its qubit (it commutes with
+// controls and other diagonals, and the gradient term of a generator Z does
+// not change across an op that commutes with it); groups are placed where the
+// most of them meet: at the end of the range that ends first, with every op
+// whose range holds that place.  A diagonal alone stays where it was.  (20
+// qubits, 10 layers of RY and RZ, 64 states: reverse passes 4.1 instead of 4.6
+// ms a segment of two layers, forward passes 1.93 instead of 2.2.)
+void group_diagonals(const std::vector<BOp>& ops, std::vector<BOp>& out) {
+  const int n = (int)ops.size();
+  struct Range {
+    int op, first, last;  // places: before op `first` .. before op `last`
+  };
+  std::vector<Range> cand;
+  auto targets = [&](int j, int q) {
+    if (ops[j].kind == OPK_DIAG) return false;
+    for (int i = 0; i < ops[j].k; i++)
+      if (ops[j].gq[i] == q) return true;
+    return false;
+  };
+  for (int i = 0; i < n; i++) {
+    const BOp& z = ops[i];
+    if (z.kind != OPK_DIAG || z.k != 1 || z.lmask || z.xmask || (z.grad && !(z.flags & OPF_GZ))) continue;
+    Range r{i, 0, n};
+    for (int j = i - 1; j >= 0 && !r.first; j--)
+      if (targets(j, z.gq[0])) r.first = j + 1;
+    for (int j = i + 1; j < n && r.last == n; j++)
+      if (targets(j, z.gq[0])) r.last = j;
+    cand.push_back(r);
+  }
+  std::stable_sort(cand.begin(), cand.end(), [](const Range& a, const Range& b) { return a.last < b.last; });
+  std::vector<char> in_group(n, 0), used(cand.size(), 0);
+  std::vector<std::vector<int>> at(n + 1);  // the members of the group placed before each op
+  for (size_t a = 0; a < cand.size(); a++) {
+    if (used[a]) continue;
+    std::vector<int> m;
+    for (size_t b = a; b < cand.size(); b++)
+      if (!used[b] && cand[b].first <= cand[a].last) m.push_back((int)b);
+    if (m.size() < 2 || !at[cand[a].last].empty()) continue;
+    for (int b : m) {
+      used[b] = 1;
+      in_group[cand[b].op] = 1;
+      at[cand[a].last].push_back(cand[b].op);
+    }
+  }
+  for (int i = 0; i <= n; i++) {
+    if (!at[i].empty()) {
+      BOp g;
+      std::memset(&g, 0, sizeof(g));
+      g.kind = OPK_ZGROUP;
+      g.k = (uint8_t)at[i].size();
+      for (int o : at[i]) g.grad |= ops[o].grad;
+      out.push_back(g);
+      for (int o : at[i]) out.push_back(ops[o]);
+    }
+    if (i < n && !in_group[i]) out.push_back(ops[i]);
+  }
+}
+
 template <typename R>
 void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, const Sweep& sw, int n, int batch,
                   int npg, bool reverse, BatchProgram<R>& P) {
@@ -227,9 +287,31 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
     return at;
   };
   if ((int)sw.ops.size() > kBatchOps) fail(SV_ERR_INVALID, "internal: too many ops in a batch program");
+  // The ops ordered by register phases, where that takes fewer of them: a
+  // phase costs its amplitudes' trip through shared memory and a barrier.  An
+  // op only passes ops it commutes with, generator included, so its gradient
+  // term is the same.  (20 qubits, 10 layers of RY, RZ and a CNOT ring, 64
+  // states: 13 forward and 11 reverse phases a segment of two layers instead of
+  // 21 and 22, 31.2 ms a gradient batch became 26.6.)
+  std::vector<int> oplist = sw.ops;
+  if (sw.m >= kRegQ && sw.m - kRegQ <= 8) {
+    std::vector<PhaseOp> pops(oplist.size());
+    for (size_t i = 0; i < oplist.size(); i++) {
+      const LOp& op = ag[order[oplist[i]]].op;
+      uint32_t nd = 0;
+      if (op.kind != OPK_DIAG)
+        for (int q = 0; q < op.k; q++)
+          if (loc[op.q[q]] >= 0) nd |= 1u << loc[op.q[q]];
+      pops[i] = phase_op(op, nd, false);
+    }
+    int phases = 0, runs = 0;
+    const std::vector<int> seq = order_by_phase(pops, kRegQ, &phases, &runs);
+    if (phases < runs)
+      for (size_t i = 0; i < seq.size(); i++) oplist[i] = sw.ops[seq[i]];
+  }
   std::vector<uint32_t> need(sw.ops.size(), 0);
   for (size_t oi = 0; oi < sw.ops.size(); oi++) {
-    const AGate& g = ag[order[sw.ops[oi]]];
+    const AGate& g = ag[order[oplist[oi]]];
     const LOp& op = g.op;
     BOp d;
     std::memset(&d, 0, sizeof(d));
@@ -288,20 +370,6 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
     }
     P.ops[oi] = d;
   }
-  P.h.nops = (int)sw.ops.size();
-  P.h.ngacc = nacc;
-  // offsets of each op's matrix and generator in the CTA's shared copy
-  int soff = 0;
-  for (int o = 0; o < P.h.nops; o++) {
-    BOp& d = P.ops[o];
-    const int dd = 1 << d.k;
-    const int mc = d.kind == OPK_DIAG ? dd : d.kind == OPK_ANTIDIAG ? 2 : d.kind == OPK_SWAP ? 0 : dd * dd;
-    const int gc = d.grad ? (d.kind == OPK_DIAG ? dd : dd * dd) : 0;
-    d.soff = (uint16_t)soff;
-    soff += mc + gc;
-  }
-  P.h.scoef = soff;
-
   // phases: consecutive ops whose moving qubits fit four register slots; tiles
   // of fewer than four qubits run every op in shared memory
   const bool reg_ok = sw.m >= kRegQ && sw.m - kRegQ <= 8;
@@ -365,6 +433,42 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
   }
   if (cur_n) add_phase(PH_REG, cur_first, cur_n, cur_need);
   P.h.nphases = nph;
+
+  // one-qubit diagonals of a register phase in groups (OPK_ZGROUP)
+  std::vector<BOp> fin;
+  for (int p = 0; p < nph; p++) {
+    Phase& ph = P.ph[p];
+    const std::vector<BOp> list(P.ops + ph.first, P.ops + ph.first + ph.nops);
+    const size_t at = fin.size();
+    if (ph.kind == PH_REG)
+      group_diagonals(list, fin);
+    else
+      fin.insert(fin.end(), list.begin(), list.end());
+    ph.first = (uint8_t)at;
+    ph.nops = (uint8_t)(fin.size() - at);
+  }
+  if ((int)fin.size() > kBatchOps) fail(SV_ERR_INVALID, "internal: too many ops in a batch program");
+  std::copy(fin.begin(), fin.end(), P.ops);
+  P.h.nops = (int)fin.size();
+  P.h.ngacc = nacc;
+  // offsets of each op's matrix and generator in the CTA's shared copy, and of
+  // each group's table (16-byte aligned)
+  int soff = 0;
+  for (int o = 0; o < P.h.nops; o++) {
+    BOp& d = P.ops[o];
+    if (d.kind == OPK_ZGROUP) {
+      soff = (soff + 1) / 2 * 2;
+      d.soff = (uint16_t)soff;
+      soff += 1 << kRegQ;
+      continue;
+    }
+    const int dd = 1 << d.k;
+    const int mc = d.kind == OPK_DIAG ? dd : d.kind == OPK_ANTIDIAG ? 2 : d.kind == OPK_SWAP ? 0 : dd * dd;
+    const int gc = d.grad ? (d.kind == OPK_DIAG ? dd : dd * dd) : 0;
+    d.soff = (uint16_t)soff;
+    soff += mc + gc;
+  }
+  P.h.scoef = soff;
 }
 
 // The batched programs of gates [g0, g1) of a template, one per pass over the
@@ -387,7 +491,7 @@ void segment_programs(const AdjTemplate& T, size_t g0, size_t g1, bool reverse, 
       ops.push_back(T.ag[i].op);
     }
   }
-  std::vector<Sweep> sws = schedule_sweeps(n, ops, tile_q, low_q, BatchProgram<R>::kPool / 2, 64, false);
+  std::vector<Sweep> sws = schedule_sweeps(n, ops, tile_q, low_q, BatchProgram<R>::kPool / 2, 64, true);
   for (const Sweep& sw : sws) {
     fill_program<R>(T.ag, order, sw, n, batch, T.npg, reverse, prog);
     each(prog);
@@ -512,7 +616,8 @@ void run_adjoint(int n, sv_dtype dtype, const sv_gate* gates, size_t ng, const d
   const int nck = ng > 0 ? (int)((ng - 1) / c) : 0;  // stored states after c, 2c, ... gates
   const int tile_q = adjoint_tile_q(dtype), low_q = low_qubits_for(dtype);
   const int m = std::min(n, tile_q);
-  const int grid_x = batch_grid_x(n, m, batch);
+  const int grid_f = batch_grid_x(n, m, batch, batch_resident(sizeof(R), false));  // CTAs per state: forward passes,
+  const int grid_x = batch_grid_x(n, m, batch, batch_resident(sizeof(R), true));   // reverse passes
   Cx<R>* psi = (Cx<R>*)scratch_buffer(stream, "adj_psi", sbytes);
   Cx<R>* lam = (Cx<R>*)scratch_buffer(stream, "adj_lam", sbytes);
   // boundaries j = 1..nck (the state after j*c gates); kept ones get a slot
@@ -559,7 +664,7 @@ void run_adjoint(int n, sv_dtype dtype, const sv_gate* gates, size_t ng, const d
     const JitKernel* k = jit ? jit_batch_lookup<R>(P, rev) : nullptr;
     Prof pr(stream, rev ? (k ? "batch_sweep_rev_jit" : "batch_sweep_rev") : (k ? "batch_sweep_fwd_jit" : "batch_sweep_fwd"),
             rev ? sweep_bytes_r : sweep_bytes_f);
-    cuda_check(launch_batch_sweep<R>(psi, rev ? lam : nullptr, dtab, gscr, grid_x, P, rev, stream, k),
+    cuda_check(launch_batch_sweep<R>(psi, rev ? lam : nullptr, dtab, gscr, rev ? grid_x : grid_f, P, rev, stream, k),
                rev ? "reverse sweep" : "forward sweep");
     pr.done();
   };

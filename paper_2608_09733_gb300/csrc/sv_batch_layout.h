@@ -49,6 +49,15 @@ struct BOp {
 };
 static_assert(sizeof(BOp) == 64, "BOp layout");
 
+// A group of uncontrolled one-qubit diagonals of a register phase (RZ of any
+// qubits, S, T ...): a header of this kind with k = the members, which follow
+// it as ops of their own.  Members on register slots make one table of 2^kRegQ
+// factors per state (at the header's soff), the others one factor a thread, so
+// psi and lambda are multiplied once for the whole group, and the gradient
+// terms of all members are signed sums of one Im(conj(lambda) psi) per
+// amplitude.  The header's grad is set when a member's is.
+constexpr uint8_t OPK_ZGROUP = 9;
+
 constexpr int kBatchOps = 96;
 constexpr int kBatchGacc = 64;   // gradient accumulators per program
 constexpr int kTableStride = 16; // complex entries per (gate, state) table row
@@ -59,6 +68,10 @@ struct BatchHeader {
   int32_t scoef, pad;  // complex entries of the shared coefficient copy
   int8_t tq[16];
 };
+
+// Resident CTAs an SM of a batched sweep (launch bounds; 256 threads).  The
+// reverse passes hold psi and lambda: two CTAs at 128 registers in complex64.
+constexpr int batch_resident(int real_bytes, bool reverse) { return real_bytes == 8 ? 1 : reverse ? 2 : 3; }
 
 template <typename R>
 struct BatchProgram {

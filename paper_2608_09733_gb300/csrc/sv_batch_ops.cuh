@@ -609,12 +609,37 @@ __device__ __forceinline__ void batch_sweep_body(Cx<R>* __restrict__ psi, Cx<R>*
   for (int o = warp; o < h.nops; o += (int)(blockDim.x >> 5)) {
     const BOp& op = P.ops[o];
     const int dd = 1 << op.k;
+    if (op.kind == OPK_ZGROUP) continue;
     const int mc = op.kind == OPK_DIAG ? dd : op.kind == OPK_ANTIDIAG ? 2 : op.kind == OPK_SWAP ? 0 : dd * dd;
     const int gc = op.grad ? (op.kind == OPK_DIAG ? dd : dd * dd) : 0;
     const Cx<R>* src = op.table ? table + ((uint64_t)op.coef * h.batch + bidx) * kTableStride : P.pool + op.coef;
     for (int e = lane; e < mc + gc; e += 32) scoef[op.soff + e] = e < mc ? src[e] : P.pool[op.gen + (e - mc)];
   }
   const uint32_t lowmask = (1u << h.L) - 1u;
+  __syncthreads();
+  for (int o = warp; o < h.nops; o += (int)(blockDim.x >> 5)) {  // the tables of diagonal groups
+    const BOp& op = P.ops[o];
+    if (op.kind != OPK_ZGROUP || lane >= NR) continue;
+    // the product in double, brought back to modulus one (every member has it)
+    // and rounded once: a table's error is one rounding, whatever it joins
+    double tr = 1.0, ti = 0.0;
+    for (int i = 1; i <= op.k; i++) {
+      const BOp& z = P.ops[o + i];
+      if (z.rs[0] == 0xFF) continue;
+      const Cx<R> u = scoef[z.soff + ((lane >> z.rs[0]) & 1)];
+      const double ur = (double)u.re, ui = z.dagger ? -(double)u.im : (double)u.im;
+      const double r = fma(tr, ur, -(ti * ui));
+      ti = fma(tr, ui, ti * ur);
+      tr = r;
+    }
+    if (sizeof(R) == 4) {
+      const double g = fma(-0.5, fma(tr, tr, ti * ti), 1.5);  // 1 / |t| for |t| close to 1
+      tr *= g;
+      ti *= g;
+    }
+    const Cx<R> t = {(R)tr, (R)ti};
+    scoef[op.soff + lane] = t;
+  }
   __syncthreads();
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     uint64_t base = tile;
@@ -625,6 +650,18 @@ __device__ __forceinline__ void batch_sweep_body(Cx<R>* __restrict__ psi, Cx<R>*
       const uint64_t off = base + (hi_off[l >> h.L] | (l & lowmask));
       cp_async16(sp + sw<R>(l), ps + off);
       if (REV) cp_async16(sl + sw<R>(l), ls + off);
+    }
+    // the next tile's lines start for L2 while this tile is worked on (a 4096-
+    // amplitude tile gathers 256-byte runs; its copies then wait for L2 only)
+    const uint64_t next = tile + gridDim.x;
+    if (next < ntiles) {
+      uint64_t nb = next;
+      for (int i = 0; i < h.m; i++) nb = ins0_64(nb, h.tq[i]);
+      for (int v = threadIdx.x * (128 / (int)sizeof(Cx<R>)); v < tsz; v += blockDim.x * (128 / (int)sizeof(Cx<R>))) {
+        const uint64_t off = nb + (hi_off[v >> h.L] | ((uint32_t)v & lowmask));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(ps + off));
+        if (REV) asm volatile("prefetch.global.L2 [%0];" ::"l"(ls + off));
+      }
     }
     cp_async_commit_wait_all();
     __syncthreads();
@@ -640,7 +677,7 @@ __device__ __forceinline__ void batch_sweep_body(Cx<R>* __restrict__ psi, Cx<R>*
   if (REV) {
     for (int o = threadIdx.x; o < h.nops; o += blockDim.x) {
       const BOp& op = P.ops[o];
-      if (!op.grad) continue;
+      if (!op.grad || op.kind == OPK_ZGROUP) continue;
       double s2 = 0.0;
       for (int w = 0; w < (int)(blockDim.x >> 5); w++) s2 += gacc[op.gacc][w];
       gscratch[((uint64_t)bidx * h.ngrad_total + op.gidx) * gridDim.x + blockIdx.x] = s2;
@@ -730,6 +767,113 @@ __device__ __forceinline__ void batch_grad_add(R acc, double* row, int warp, int
   if (lane == 0) row[warp] += (double)w;
 }
 
+// Four gradient terms at once: the warp's sums by halving exchanges (six
+// shuffles, not twenty), then added in double by four lanes, one term each.
+template <typename R>
+__device__ __forceinline__ void batch_grad_add4(const R (&a)[4], int r0, int r1, int r2, int r3, int count,
+                                                double (*gacc)[8], int warp, int lane) {
+  const bool h16 = lane & 16, h8 = lane & 8;
+  R b0 = (h16 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, h16 ? a[0] : a[2], 16);
+  R b1 = (h16 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, h16 ? a[1] : a[3], 16);
+  R c = (h8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h8 ? b0 : b1, 8);
+#pragma unroll
+  for (int s2 = 4; s2 > 0; s2 >>= 1) c += __shfl_xor_sync(0xffffffffu, c, s2);
+  const int which = lane >> 3;
+  if ((lane & 7) == 0 && which < count)
+    gacc[which == 0 ? r0 : which == 1 ? r1 : which == 2 ? r2 : r3][warp] += (double)c;
+}
+
+// A diagonal group on the thread's registers: amplitude j of psi and lambda
+// times T[j] (times the thread's factor f with HASF).  With GR, before that,
+// w_j = Im(conj(lambda_j) psi_j) and its sums: t0 over all j, d[s] over the j
+// with slot s clear less those with it set, pairwise over the slots (30 adds
+// for all four and the total).
+template <typename R, bool REV, bool HASF, bool GR>
+__device__ __forceinline__ void batch_z_apply(Cx<R> (&p)[NR], Cx<R> (&l)[NR], const Cx<R>* T, Cx<R> f, R (&d)[kRegQ],
+                                              R& t0) {
+  if constexpr (REV && GR) {
+    R w[NR];
+#pragma unroll
+    for (int j = 0; j < NR; j++) w[j] = im_cdot(l[j], p[j]);
+#pragma unroll
+    for (int s = 0; s < kRegQ; s++) {
+      R x = R(0);
+#pragma unroll
+      for (int i = 0; i < (NR >> (s + 1)); i++) {
+        x += w[2 * i] - w[2 * i + 1];
+        w[i] = w[2 * i] + w[2 * i + 1];
+      }
+      d[s] = x;
+    }
+    t0 = w[0];
+  }
+#pragma unroll
+  for (int j = 0; j < NR; j++) {
+    Cx<R> t = T[j];
+    if (HASF) t = cmul(f, t);
+    p[j] = cmul(t, p[j]);
+    if (REV) l[j] = cmul(t, l[j]);
+  }
+}
+
+// The group with header g[0] and members g[1 .. g[0].k].
+template <typename R, bool REV>
+__device__ __forceinline__ void batch_zgroup(const BOp* g, Cx<R> (&p)[NR], Cx<R> (&l)[NR], uint32_t tb, bool active,
+                                             const Cx<R>* scoef, uint64_t base, double (*gacc)[8], int warp,
+                                             int lane) {
+  Cx<R> f = {R(1), R(0)};
+  bool has = false;
+  auto fixed_bit = [&](const BOp& z) {
+    return z.pos[0] != 0xFF ? (tb >> z.pos[0]) & 1u : (uint32_t)(base >> z.gq[0]) & 1u;
+  };
+  for (int i = 1; i <= g->k; i++) {
+    if (g[i].rs[0] != 0xFF) continue;
+    const Cx<R> m = scoef[g[i].soff + fixed_bit(g[i])];
+    const Cx<R> u = g[i].dagger ? conjx(m) : m;
+    f = has ? cmul(f, u) : u;
+    has = true;
+  }
+  R d[kRegQ] = {R(0), R(0), R(0), R(0)}, t0 = R(0);
+  const bool grad = REV && g->grad;
+  const Cx<R>* T = scoef + g->soff;
+  if (active) {
+    if (has) {
+      if (grad)
+        batch_z_apply<R, REV, true, true>(p, l, T, f, d, t0);
+      else
+        batch_z_apply<R, REV, true, false>(p, l, T, f, d, t0);
+    } else {
+      if (grad)
+        batch_z_apply<R, REV, false, true>(p, l, T, f, d, t0);
+      else
+        batch_z_apply<R, REV, false, false>(p, l, T, f, d, t0);
+    }
+  }
+  if (!grad) return;
+  R a[4] = {R(0), R(0), R(0), R(0)};
+  int r[4] = {0, 0, 0, 0}, n = 0;
+  for (int i = 1; i <= g->k; i++) {
+    const BOp& z = g[i];
+    if (!z.grad) continue;
+    const R v = z.rs[0] == 0 ? d[0] : z.rs[0] == 1 ? d[1] : z.rs[0] == 2 ? d[2] : z.rs[0] == 3 ? d[3]
+                : fixed_bit(z) ? -t0 : t0;
+    a[0] = n == 0 ? v : a[0];
+    a[1] = n == 1 ? v : a[1];
+    a[2] = n == 2 ? v : a[2];
+    a[3] = n == 3 ? v : a[3];
+    r[0] = n == 0 ? z.gacc : r[0];
+    r[1] = n == 1 ? z.gacc : r[1];
+    r[2] = n == 2 ? z.gacc : r[2];
+    r[3] = n == 3 ? z.gacc : r[3];
+    if (++n == 4) {
+      batch_grad_add4<R>(a, r[0], r[1], r[2], r[3], 4, gacc, warp, lane);
+      n = 0;
+      a[0] = a[1] = a[2] = a[3] = R(0);
+    }
+  }
+  if (n) batch_grad_add4<R>(a, r[0], r[1], r[2], r[3], n, gacc, warp, lane);
+}
+
 // One op of a register phase on the thread's registers (when the op's
 // controls on the tile's and the thread's fixed bits hold), then, for a
 // gradient op, the warp's sum of its term in the state's precision added in
@@ -789,8 +933,14 @@ struct BatchInterp {
       const Phase& ph = P.ph[ph_i];
       if (ph.kind == PH_REG) {
         batch_reg_phase<R, REV>(ph, sp, sl, [&](Cx<R>(&p)[NR], Cx<R>(&l)[NR], uint32_t tb, bool active) {
-          for (int o = ph.first; o < ph.first + ph.nops; o++)
-            batch_reg_op<R, REV>(P.ops[o], p, l, tb, active, scoef, base, gacc, warp, lane);
+          for (int o = ph.first; o < ph.first + ph.nops; o++) {
+            if (P.ops[o].kind == OPK_ZGROUP) {
+              batch_zgroup<R, REV>(P.ops + o, p, l, tb, active, scoef, base, gacc, warp, lane);
+              o += P.ops[o].k;
+            } else {
+              batch_reg_op<R, REV>(P.ops[o], p, l, tb, active, scoef, base, gacc, warp, lane);
+            }
+          }
         });
       } else {
         batch_smem_op<R, REV>(P.ops[ph.first], sp, sl, tsz, scoef, base, gacc, warp, lane);

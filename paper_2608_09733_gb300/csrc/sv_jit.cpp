@@ -580,6 +580,64 @@ std::string batch_reg_call(const BOp& d, bool rev, const char* Rn) {
   }
 }
 
+// batch_zgroup (sv_batch_ops.cuh) of the group with header g[0], its members
+// as constants.
+void emit_zgroup(Src& o, const BOp* g, bool rev, const char* Rn) {
+  const bool grad = rev && g->grad;
+  auto bit = [](const BOp& z) {
+    char b[64];
+    if (z.pos[0] != 0xFF)
+      snprintf(b, sizeof(b), "((tb >> %d) & 1u)", z.pos[0]);
+    else
+      snprintf(b, sizeof(b), "((uint32_t)(base >> %d) & 1u)", z.gq[0]);
+    return std::string(b);
+  };
+  o.line("      {  // %d one-qubit diagonals", g->k);
+  bool has = false;
+  o.line("        Cx<%s> f = {%s(1), %s(0)};", Rn, Rn, Rn);
+  for (int i = 1; i <= g->k; i++) {
+    const BOp& z = g[i];
+    if (z.rs[0] != 0xFF) continue;
+    char u[128];
+    snprintf(u, sizeof(u), z.dagger ? "conjx(scoef[%u + %s])" : "scoef[%u + %s]", (unsigned)z.soff, bit(z).c_str());
+    if (has)
+      o.line("        f = cmul(f, %s);", u);
+    else
+      o.line("        f = %s;", u);
+    has = true;
+  }
+  o.line("        %s d[kRegQ] = {%s(0), %s(0), %s(0), %s(0)}, t0 = %s(0);", Rn, Rn, Rn, Rn, Rn, Rn);
+  o.line("        if (active) batch_z_apply<%s, %s, %s, %s>(p, l, scoef + %u, f, d, t0);", Rn, rev ? "true" : "false",
+         has ? "true" : "false", grad ? "true" : "false", (unsigned)g->soff);
+  if (grad) {
+    std::vector<std::string> v;
+    std::vector<int> r;
+    auto flush = [&] {
+      if (v.empty()) return;
+      const int n = (int)v.size();
+      while (v.size() < 4) {
+        v.push_back(std::string(Rn) + "(0)");
+        r.push_back(0);
+      }
+      o.line("        {");
+      o.line("          const %s a[4] = {%s, %s, %s, %s};", Rn, v[0].c_str(), v[1].c_str(), v[2].c_str(), v[3].c_str());
+      o.line("          batch_grad_add4<%s>(a, %d, %d, %d, %d, %d, gacc, warp, lane);", Rn, r[0], r[1], r[2], r[3], n);
+      o.line("        }");
+      v.clear();
+      r.clear();
+    };
+    for (int i = 1; i <= g->k; i++) {
+      const BOp& z = g[i];
+      if (!z.grad) continue;
+      v.push_back(z.rs[0] != 0xFF ? "d[" + std::to_string(z.rs[0]) + "]" : "(" + bit(z) + " ? -t0 : t0)");
+      r.push_back(z.gacc);
+      if (v.size() == 4) flush();
+    }
+    flush();
+  }
+  o.line("      }");
+}
+
 }  // namespace
 
 // The kernel source of one batched adjoint program: every phase and op as a
@@ -608,6 +666,11 @@ std::string jit_batch_source(const BatchProgram<R>& P, bool rev) {
         // batch_reg_op of the interpreting kernel, its dispatch and
         // conditions decided here
         const BOp& d = P.ops[ph.first + i];
+        if (d.kind == OPK_ZGROUP) {
+          emit_zgroup(o, &d, rev, Rn);
+          i += d.k;
+          continue;
+        }
         const int dd = 1 << d.k;
         std::string cond = "active";
         char cb[160];
@@ -645,7 +708,7 @@ std::string jit_batch_source(const BatchProgram<R>& P, bool rev) {
   o.line("  }");
   o.line("};");
   o.line("}  // namespace sv");
-  o.line("extern \"C\" __global__ void __launch_bounds__(256, %d)", sizeof(R) == 4 ? 2 : 1);
+  o.line("extern \"C\" __global__ void __launch_bounds__(256, %d)", batch_resident(sizeof(R), rev));
   o.line("k_batch_sweep_jit(sv::Cx<%s>* __restrict__ psi, sv::Cx<%s>* __restrict__ lam,", Rn, Rn);
   o.line("                  const sv::Cx<%s>* __restrict__ table, double* __restrict__ gscratch,", Rn);
   o.line("                  const __grid_constant__ sv::BatchProgram<%s> P) {", Rn);

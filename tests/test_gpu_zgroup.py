@@ -1,0 +1,66 @@
+"""Groups of one-qubit diagonals in the batched adjoint passes, against the
+oracle's gradients: several rotations of one qubit, members on register slots,
+thread bits and bits outside the tile, more than four gradient members,
+constant diagonals, and diagonals that must stay out (controls, generators
+other than Z); compiled and interpreted passes give the same bits."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2608_09733_gb300 as sv
+from workloads import Gate, Term
+
+pytestmark = pytest.mark.gpu
+
+TOL = {sv.SV_C64: 1e-4, sv.SV_C128: 1e-10}  # the gradient tolerances of the other adjoint tests
+
+
+def _template(n, layers, seed):
+    rng = np.random.default_rng(seed)
+    gates, slot = [], 0
+
+    def rot(name, targets, controls=()):
+        nonlocal slot
+        gates.append(Gate(name, list(targets), list(controls), slots=[slot], params=[0.0]))
+        slot += 1
+
+    for _ in range(layers):
+        for q in range(n):
+            if rng.integers(3):
+                rot("ry", [q])
+            for _ in range(int(rng.integers(0, 3))):
+                rot("rz", [q])
+            if not rng.integers(4):
+                gates.append(Gate(["s", "t", "z"][int(rng.integers(3))], [q]))
+        for q in range(n):
+            other = (q + 1 + int(rng.integers(n - 1))) % n
+            kind = rng.integers(6)
+            if kind < 2:
+                gates.append(Gate("x", [other], [q]))
+            elif kind == 2:
+                rot("rz", [other], [q])
+            elif kind == 3:
+                rot("p", [q])
+            elif kind == 4:
+                rot("rzz", [q, other])
+    return gates, slot
+
+
+@pytest.mark.parametrize("dtype", [sv.SV_C64, sv.SV_C128])
+@pytest.mark.parametrize("n,layers,ckpt", [(3, 3, 0), (4, 2, 0), (6, 3, 10), (13, 2, 0), (14, 2, 25)])
+def test_gradients(svlib, cuda_dev, n, layers, ckpt, dtype):
+    gates, npar = _template(n, layers, seed=n)
+    terms = [Term("Z", [q], 1.0) for q in range(n)] + [Term("X", [0], 0.5), Term("XY", [0, n - 1], 0.3)]
+    th = np.random.default_rng(n).uniform(-np.pi, np.pi, size=(3, npar))
+    out = []
+    try:
+        for mode in (0, 2):
+            sv.sv_jit_set_mode(mode)
+            out.append(sv.sv_adjoint_grad(n, dtype, gates, th, terms, checkpoint_every=ckpt))
+    finally:
+        sv.sv_jit_set_mode(-1)
+    (v, g), (v2, g2) = out
+    assert np.array_equal(v, v2) and np.array_equal(g, g2)
+    for b in range(3):
+        v_ref, g_ref = oracle.adjoint_grad(n, gates, th[b], terms, npar)
+        assert abs(v[b] - v_ref) < TOL[dtype] and np.abs(g[b] - g_ref).max() < TOL[dtype]
