@@ -101,7 +101,11 @@ struct PauliTilePass {
   uint16_t orig[kPauliTileTerms];     // the term's index in the caller's list (per-state coefficients)
   uint8_t ny[kPauliTileTerms];        // nY_j mod 4
   int32_t nterms_all;                 // terms per state in the per-state coefficient rows
+  // the first nlow terms have no X and Z only on local bits below kPauliLowBits,
+  // the next nhigh no X and Z on none of those
+  int32_t nlow, nhigh;
 };
+constexpr int kPauliLowBits = 7;
 
 // The pass's coefficients in the state's precision (FP64 is a slow pipe on
 // GB300), staged in shared memory by the kernel.
@@ -112,6 +116,13 @@ struct PauliTileCoef {
 
 // With `rowc` (device, batch x nterms_all doubles) state b takes its own
 // coefficients c_{b,j} in place of P.cr / P.ci.
+//
+// The sum was bound by the signs of its terms: a ring of 20 ZZ and 20 X terms
+// cost each amplitude 40 popcounts and selects (64 states of 20 qubits: 2.3
+// ms).  Z terms within the low or the high local bits of the tile are summed
+// once per tile into two tables, tl by the low bits and th by the high ones,
+// and a term alone on its X mask without local Z takes its sign per tile: the
+// same sum in 1.6 ms (HBM alone: 0.4).
 template <typename R>
 __global__ void __launch_bounds__(256) k_pauli_tiles(const Cx<R>* __restrict__ psi, Cx<R>* __restrict__ lam,
                                                      const __grid_constant__ PauliTilePass P, uint64_t ntiles,
@@ -125,9 +136,11 @@ __global__ void __launch_bounds__(256) k_pauli_tiles(const Cx<R>* __restrict__ p
   // the terms' masks, staged once (broadcast reads in the inner loop)
   // The sign (-1)^{popc((g ^ x) & z)} of a term splits into the tile-local
   // part popc(l & zl) and a part that is fixed over the tile (the bits
-  // outside it, and x inside it): sc0[j], restaged per tile.
+  // outside it, and x inside it), which scf[j] holds.
   __shared__ uint32_t sxl[kPauliTileTerms], szl[kPauliTileTerms];
-  __shared__ uint8_t sgend[kPauliTileTerms], sc0[kPauliTileTerms];
+  __shared__ uint8_t sgend[kPauliTileTerms];
+  __shared__ PauliTileCoef<R> scf[kPauliTileTerms];  // the coefficients with the tile's signs
+  __shared__ R tl[1 << kPauliLowBits], th[1 << (14 - kPauliLowBits)];
   for (int j = threadIdx.x; j < P.nterms; j += blockDim.x) {
     sxl[j] = P.xl[j];
     szl[j] = P.zl[j];
@@ -162,9 +175,29 @@ __global__ void __launch_bounds__(256) k_pauli_tiles(const Cx<R>* __restrict__ p
     }
     for (int l = threadIdx.x; l < tsz; l += blockDim.x)
       s[l] = psi[sbase + (base | hi_off[l >> P.L] | (l & lowmask))];
-    for (int j = threadIdx.x; j < P.nterms; j += blockDim.x)
-      sc0[j] = (uint8_t)((__popcll((base ^ P.xg[j]) & P.z[j] & ~tile_mask) + __popc(P.xl[j] & P.zl[j])) & 1);
+    if (rowc) __syncthreads();  // cf of this state
+    for (int j = threadIdx.x; j < P.nterms; j += blockDim.x) {
+      const bool neg = (__popcll((base ^ P.xg[j]) & P.z[j] & ~tile_mask) + __popc(P.xl[j] & P.zl[j])) & 1;
+      const PauliTileCoef<R> c = cf[j];
+      scf[j] = neg ? PauliTileCoef<R>{-c.cr, -c.ci} : c;
+    }
     __syncthreads();
+    const int ndiag = P.nlow + P.nhigh;
+    if (ndiag) {
+      const int high = 1 << (P.m > kPauliLowBits ? P.m - kPauliLowBits : 0);
+      for (int e = threadIdx.x; e < (1 << kPauliLowBits) + high; e += blockDim.x) {
+        const bool is_high = e >= (1 << kPauliLowBits);
+        const uint32_t l = is_high ? (uint32_t)(e - (1 << kPauliLowBits)) << kPauliLowBits : (uint32_t)e;
+        R sum = R(0);
+        for (int j = is_high ? P.nlow : 0; j < (is_high ? ndiag : P.nlow); j++)
+          sum += (__popc(l & szl[j]) & 1) ? -scf[j].cr : scf[j].cr;
+        if (is_high)
+          th[e - (1 << kPauliLowBits)] = sum;
+        else
+          tl[e] = sum;
+      }
+      __syncthreads();
+    }
     // four amplitudes per thread: each term's masks and coefficient are read
     // once for all four, and the four sums are independent
     constexpr int A = 4;
@@ -184,15 +217,31 @@ __global__ void __launch_bounds__(256) k_pauli_tiles(const Cx<R>* __restrict__ p
       for (int j = 0; j < P.nterms;) {
         const uint32_t xl = sxl[j];
         const int je = sgend[j];
+        if (je == j + 1 && szl[j] == 0u && j >= ndiag) {  // one term, its sign fixed over the tile
+          const PauliTileCoef<R> c = scf[j];
+#pragma unroll
+          for (int k = 0; k < A; k++) {
+            const Cx<R> v = s[lk[k] ^ xl];
+            ar[k] = fma(c.cr, v.re, fma(-c.ci, v.im, ar[k]));
+            ai[k] = fma(c.cr, v.im, fma(c.ci, v.re, ai[k]));
+          }
+          j = je;
+          continue;
+        }
         R fr[A], fi[A];
 #pragma unroll
         for (int k = 0; k < A; k++) fr[k] = fi[k] = R(0);
+        if (j < ndiag) {  // the terms without X begin with the tabled ones
+#pragma unroll
+          for (int k = 0; k < A; k++) fr[k] = tl[lk[k] & ((1 << kPauliLowBits) - 1)] + th[lk[k] >> kPauliLowBits];
+          j = ndiag;
+        }
         for (; j < je; j++) {
-          const uint32_t zl = szl[j], c0 = sc0[j];
-          const PauliTileCoef<R> c = cf[j];
+          const uint32_t zl = szl[j];
+          const PauliTileCoef<R> c = scf[j];
 #pragma unroll
           for (int k = 0; k < A; k++) {
-            const bool neg = (__popc((uint32_t)lk[k] & zl) ^ c0) & 1u;
+            const bool neg = __popc((uint32_t)lk[k] & zl) & 1u;
             fr[k] += neg ? -c.cr : c.cr;
             fi[k] += neg ? -c.ci : c.ci;
           }
@@ -401,11 +450,30 @@ cudaError_t launch_pauli_tiles(const Cx<R>* psi, Cx<R>* lam, int n, int batch, c
       if (grid > ntiles) grid = ntiles;
       k_pauli_tiles<R><<<(unsigned)grid, 256, smem, stream>>>(psi, lam, P, ntiles, rowc);
       acc = true;
-      P.nterms = 0;
+      P.nterms = P.nlow = P.nhigh = 0;
       return cudaGetLastError();
     };
-    for (int t : idx) {
-      if (done[t] || (terms[t].x_mask & ~T)) continue;
+    // the pass's terms by X mask; those without X whose Z is within the low or
+    // the high local bits first
+    std::vector<int> pass_terms;
+    auto local_z = [&](int t) {
+      uint32_t zl = 0;
+      for (int q = 0; q < n; q++)
+        if (((terms[t].z_mask >> q) & 1ull) && ((T >> q) & 1ull)) zl |= 1u << loc[q];
+      return zl;
+    };
+    const uint32_t low_bits = (1u << kPauliLowBits) - 1u;
+    auto kind_of = [&](int t) {  // 0 low, 1 high, 2 neither
+      if (terms[t].x_mask) return 2;
+      const uint32_t zl = local_z(t);
+      return !(zl & ~low_bits) ? 0 : !(zl & low_bits) ? 1 : 2;
+    };
+    for (int t : idx)
+      if (!done[t] && !(terms[t].x_mask & ~T)) pass_terms.push_back(t);
+    std::stable_sort(pass_terms.begin(), pass_terms.end(), [&](int a, int b) {
+      return terms[a].x_mask != terms[b].x_mask ? terms[a].x_mask < terms[b].x_mask : kind_of(a) < kind_of(b);
+    });
+    for (int t : pass_terms) {
       if (P.nterms == kPauliTileTerms) {
         cudaError_t e = flush();
         if (e != cudaSuccess) return e;
@@ -420,10 +488,9 @@ cudaError_t launch_pauli_tiles(const Cx<R>* psi, Cx<R>* lam, int n, int batch, c
       P.xl[j] = xl;
       P.xg[j] = x;
       P.z[j] = terms[t].z_mask;
-      uint32_t zl = 0;
-      for (int q = 0; q < n; q++)
-        if (((terms[t].z_mask >> q) & 1ull) && ((T >> q) & 1ull)) zl |= 1u << loc[q];
-      P.zl[j] = zl;
+      P.zl[j] = local_z(t);
+      if (kind_of(t) == 0) P.nlow++;
+      if (kind_of(t) == 1) P.nhigh++;
       P.cr[j] = ny == 0 ? c : ny == 2 ? -c : 0.0;
       P.ci[j] = ny == 1 ? c : ny == 3 ? -c : 0.0;
       P.orig[j] = (uint16_t)t;
