@@ -280,14 +280,11 @@ std::shared_ptr<const Compiled> compiled_circuit(int n, sv_dtype dtype, const sv
   Plan plan = make_plan(n, dtype, gates, ng, pv, npv, opts, 0, lane);
   auto c = std::make_shared<Compiled>();
   c->n = n;
-  if (dtype == SV_C64) {
-    c->pf.resize(plan.sweeps.size());
-    for (size_t i = 0; i < plan.sweeps.size(); i++) build_program<float>(plan, plan.sweeps[i], c->pf[i]);
-  } else {
-    c->pd.resize(plan.sweeps.size());
-    for (size_t i = 0; i < plan.sweeps.size(); i++) build_program<double>(plan, plan.sweeps[i], c->pd[i]);
-  }
-  if (plan.sweeps.size() <= kCompiledMaxPasses) {
+  if (dtype == SV_C64)
+    build_programs<float>(plan, c->pf);
+  else
+    build_programs<double>(plan, c->pd);
+  if (c->pf.size() + c->pd.size() <= kCompiledMaxPasses) {
     c->key = std::move(key);
     std::lock_guard<std::mutex> lk(g_compiled_mu);
     g_compiled.push_front(c);
@@ -481,13 +478,21 @@ sv_status sv_plan_info(int n_qubits, sv_dtype dtype, const sv_gate* gates, size_
   return guarded([&] {
     const sv_exec_opts o = opts_of(opts);
     Plan plan = make_plan(n_qubits, dtype, gates, n_gates, param_values, n_param_values, o, 0, lane_sizes(n_qubits, o));
-    if (std::getenv("SV_DEBUG_PLAN")) {  // print the device programs (host only)
-      std::unique_ptr<SweepProgram<float>> pf(new SweepProgram<float>());
-      for (const Sweep& sw : plan.sweeps) build_program<float>(plan, sw, *pf);
+    // the passes that run: a pass of the plan can take more than one program
+    // (SV_DEBUG_PLAN prints each)
+    size_t passes = 0;
+    if (dtype == SV_C64) {
+      std::vector<SweepProgram<float>> progs;
+      build_programs<float>(plan, progs);
+      passes = progs.size();
+    } else {
+      std::vector<SweepProgram<double>> progs;
+      build_programs<double>(plan, progs);
+      passes = progs.size();
     }
     int nb = (int)plan.block_starts.size() - 1;
     if (out_blocks) *out_blocks = nb;
-    if (out_sweeps) *out_sweeps = (int)plan.sweeps.size();
+    if (out_sweeps) *out_sweeps = (int)passes;
     if (block_starts)
       for (size_t i = 0; i < plan.block_starts.size(); i++) block_starts[i] = plan.block_starts[i];
   });
@@ -677,12 +682,12 @@ void run_batch_small(int nreq, sv_dtype dtype, const int* nq, const sv_gate* con
   std::vector<Request> req(nreq);
   for_each_request(nreq, [&](int b) {
     const Plan plan = make_plan(nq[b], dtype, gates[b], ng[b], nullptr, 0, o, nq[b]);
-    std::unique_ptr<SweepProgram<R>> prog(new SweepProgram<R>());
-    for (const Sweep& sw : plan.sweeps) {
-      build_program<R>(plan, sw, *prog, kRegQ);
-      const char* p = reinterpret_cast<const char*>(prog.get());
+    std::vector<SweepProgram<R>> progs;
+    build_programs<R>(plan, progs, kRegQ);
+    for (const SweepProgram<R>& prog : progs) {
+      const char* p = reinterpret_cast<const char*>(&prog);
       req[b].offset.push_back((uint32_t)req[b].bytes.size());
-      req[b].bytes.insert(req[b].bytes.end(), p, p + staged_bytes<R>(prog->h.ncoef));
+      req[b].bytes.insert(req[b].bytes.end(), p, p + staged_bytes<R>(prog.h.ncoef));
     }
   });
   // Staging: the index (first program of each request, qubits of each request,
@@ -789,12 +794,12 @@ sv_status sv_jit_check(int n_qubits, sv_dtype dtype, const sv_gate* gates, size_
     Plan plan = make_plan(n_qubits, dtype, gates, n_gates, param_values, n_param_values, opts_of(opts));
     std::string err, src;
     if (dtype == SV_C64) {
-      std::vector<SweepProgram<float>> progs(plan.sweeps.size());
-      for (size_t i = 0; i < plan.sweeps.size(); i++) build_program<float>(plan, plan.sweeps[i], progs[i]);
+      std::vector<SweepProgram<float>> progs;
+      build_programs<float>(plan, progs);
       jit_check_programs<float>(progs, compile != 0, arch, n_sources, n_compiled, &err, &src);
     } else {
-      std::vector<SweepProgram<double>> progs(plan.sweeps.size());
-      for (size_t i = 0; i < plan.sweeps.size(); i++) build_program<double>(plan, plan.sweeps[i], progs[i]);
+      std::vector<SweepProgram<double>> progs;
+      build_programs<double>(plan, progs);
       jit_check_programs<double>(progs, compile != 0, arch, n_sources, n_compiled, &err, &src);
     }
     if (text && text_cap) {

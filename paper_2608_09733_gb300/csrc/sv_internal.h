@@ -141,8 +141,10 @@ PhaseOp phase_op(const LOp& op, uint32_t need, bool smem);
 // order, a phase ending at the first op that does not fit.
 std::vector<int> order_by_phase(const std::vector<PhaseOp>& ops, int rq, int* phases, int* runs);
 
+// The device programs of a plan's passes, appended to `out`: one a pass, more
+// where a pass does not fit one.
 template <typename R>
-void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override = 0);
+void build_programs(const Plan& plan, std::vector<SweepProgram<R>>& out, int rq_override = 0);
 
 // ----------------------------------------------------------------- launches
 // (sv_sweep.cu / sv_reduce.cu).  All return cudaError_t of the launch.

@@ -64,9 +64,11 @@ bool rot_split(const cplx* U, double tol, RotSplit& r) {
 // register slots form one register phase; dense k >= 3 blocks and wide
 // diagonals get a shared-memory phase of their own.
 // order: 0 keeps the pass's op order, 1 orders by phases where the rule below
-// says so, 2 always.
+// says so, 2 always.  False when the pass does not fit one program: the
+// scheduler counts its ops and their coefficients, not the tables, merged
+// groups and phases that are made of them here.
 template <typename R>
-void build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override, int order_by) {
+bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override, int order_by) {
   std::memset(&P.h, 0, sizeof(P.h));
   P.h.n = plan.n;
   P.h.m = sw.m;
@@ -220,8 +222,10 @@ void build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
 
   // phases
   int nph = 0;
+  bool fits = true;
   auto add_phase = [&](PhaseKind kind, int first, int nops, uint32_t need) {
-    if (nph >= kMaxPhases) fail(SV_ERR_INVALID, "internal: too many phases");
+    if (nph >= kMaxPhases) fits = false;
+    if (!fits) return;
     Phase& ph = P.ph[nph++];
     std::memset(&ph, 0, sizeof(ph));
     ph.kind = kind;
@@ -346,6 +350,7 @@ void build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
   }
   cur_n += pend;
   if (cur_n) add_phase(PH_REG, cur_first, cur_n, cur_need);
+  if (!fits) return false;
   P.h.nphases = nph;
 
   // Final op list.  In a register phase, a run of uncontrolled one-qubit
@@ -751,19 +756,19 @@ void build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
     return (int)fin.size() <= kMaxOps && ncoef <= (size_t)SweepProgram<R>::kPool;
   };
   if (!make_fin(g_rot_split, 3) && !make_fin(g_rot_split, 2) && !make_fin(g_rot_split, 0) && !make_fin(false, 0))
-    fail(SV_ERR_INVALID, "internal: program too long");
+    return false;
   P.h.nops = (int)fin.size();
 
   int coef = 0;
   for (size_t oi = 0; oi < fin.size(); oi++) {
     if (fin[oi].d.kind == OPK_PHASE && sizeof(R) == 4 && (coef & 1)) {  // tables are read in 16-byte pairs
-      if (coef >= SweepProgram<R>::kPool) fail(SV_ERR_INVALID, "internal: coefficient pool overflow");
+      if (coef >= SweepProgram<R>::kPool) return false;
       P.coef[coef].re = P.coef[coef].im = (R)0;
       coef++;
     }
     fin[oi].d.coef = (uint32_t)coef;
     for (const cplx& v : fin[oi].m) {
-      if (coef >= SweepProgram<R>::kPool) fail(SV_ERR_INVALID, "internal: coefficient pool overflow");
+      if (coef >= SweepProgram<R>::kPool) return false;
       P.coef[coef].re = (R)v.real();
       P.coef[coef].im = (R)v.imag();
       coef++;
@@ -805,17 +810,15 @@ void build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
     }
     std::fprintf(stderr, "\n");
   }
+  return true;
 }
 
 // Complex128 passes of many tiles are bound by the FP64 pipe: a table is four
 // instructions an amplitude, a phase none, so both orders are built and the
 // one with fewer tables is kept (by less than two phases a table).
 template <typename R>
-void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override) {
-  if (!(sizeof(R) == 8 && plan.carry_flips && !plan.lane)) {
-    build_program_ordered<R>(plan, sw, P, rq_override, 1);
-    return;
-  }
+bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override) {
+  if (!(sizeof(R) == 8 && plan.carry_flips && !plan.lane)) return build_program_ordered<R>(plan, sw, P, rq_override, 1);
   auto cost = [](const SweepProgram<R>& p) {
     int tables = 0;
     for (int i = 0; i < p.h.nphases; i++)
@@ -823,14 +826,37 @@ void build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
         for (int o = p.ph[i].first; o < p.ph[i].first + p.ph[i].nops; o++) tables += (p.ops[o].pad & 15u) == OPK_PHASE;
     return 2 * tables + p.h.nphases;
   };
-  build_program_ordered<R>(plan, sw, P, rq_override, 0);
   std::unique_ptr<SweepProgram<R>> other(new SweepProgram<R>());
-  build_program_ordered<R>(plan, sw, *other, rq_override, 2);
-  if (cost(*other) < cost(P)) std::memcpy(&P, other.get(), sizeof(P));
+  const bool fits = build_program_ordered<R>(plan, sw, P, rq_override, 0);
+  const bool other_fits = build_program_ordered<R>(plan, sw, *other, rq_override, 2);
+  if (other_fits && (!fits || cost(*other) < cost(P))) std::memcpy(&P, other.get(), sizeof(P));
+  return fits || other_fits;
 }
 
-template void build_program<float>(const Plan&, const Sweep&, SweepProgram<float>&, int);
-template void build_program<double>(const Plan&, const Sweep&, SweepProgram<double>&, int);
+// A pass that does not fit one program is cut in half, in its op order and with
+// the same tile, until each part does.
+template <typename R>
+static void build_parts(const Plan& plan, const Sweep& sw, std::vector<SweepProgram<R>>& out, int rq_override) {
+  out.emplace_back();
+  if (build_program<R>(plan, sw, out.back(), rq_override)) return;
+  out.pop_back();
+  if (sw.ops.size() < 2) fail(SV_ERR_INVALID, "internal: one operation does not fit a program");
+  const auto half = sw.ops.begin() + sw.ops.size() / 2;
+  Sweep part = sw;
+  part.ops.assign(sw.ops.begin(), half);
+  build_parts<R>(plan, part, out, rq_override);
+  part.ops.assign(half, sw.ops.end());
+  build_parts<R>(plan, part, out, rq_override);
+}
+
+template <typename R>
+void build_programs(const Plan& plan, std::vector<SweepProgram<R>>& out, int rq_override) {
+  out.reserve(out.size() + plan.sweeps.size());
+  for (const Sweep& sw : plan.sweeps) build_parts<R>(plan, sw, out, rq_override);
+}
+
+template void build_programs<float>(const Plan&, std::vector<SweepProgram<float>>&, int);
+template void build_programs<double>(const Plan&, std::vector<SweepProgram<double>>&, int);
 
 }  // namespace sv
 
@@ -1128,17 +1154,13 @@ extern "C" sv_status sv_emulate_apply(int n_qubits, sv_dtype dtype, const sv_gat
                                 lane_sizes(n_qubits, o));
     zc* st = reinterpret_cast<zc*>(state);
     if (dtype == SV_C64) {
-      std::unique_ptr<SweepProgram<float>> P(new SweepProgram<float>());
-      for (const Sweep& sw : plan.sweeps) {
-        build_program<float>(plan, sw, *P);
-        emulate_program<float>(*P, st);
-      }
+      std::vector<SweepProgram<float>> progs;
+      build_programs<float>(plan, progs);
+      for (const SweepProgram<float>& P : progs) emulate_program<float>(P, st);
     } else {
-      std::unique_ptr<SweepProgram<double>> P(new SweepProgram<double>());
-      for (const Sweep& sw : plan.sweeps) {
-        build_program<double>(plan, sw, *P);
-        emulate_program<double>(*P, st);
-      }
+      std::vector<SweepProgram<double>> progs;
+      build_programs<double>(plan, progs);
+      for (const SweepProgram<double>& P : progs) emulate_program<double>(P, st);
     }
   });
 }

@@ -139,9 +139,7 @@ void build_request_programs(int n, const sv_gate* gates, size_t ng, std::vector<
   // whole state in one tile: 16 amplitudes a thread up to 12 qubits, 32 at 13
   // and 14 (2^9 register groups: the session runs 512-thread CTAs for those)
   const int rq = n >= 13 ? 5 : kRegQ;
-  const size_t k0 = out.size();
-  out.resize(k0 + plan.sweeps.size());
-  for (size_t i = 0; i < plan.sweeps.size(); i++) build_program<R>(plan, plan.sweeps[i], out[k0 + i], rq);
+  build_programs<R>(plan, out, rq);
 }
 
 template <typename R>
