@@ -411,6 +411,9 @@ typedef struct sv_small_session sv_small_session;
  * programs held for them (1..65536, about 32 KB each on the device). */
 sv_status sv_small_session_start(sv_dtype dtype, int capacity, int arena_programs, double wait_limit_s, int n_ctas,
                                  sv_small_session** out);
+/* Dynamic shared memory of one session CTA in bytes (0: unknown dtype): what
+ * kernels that share its SM have to fit beside.  Needs no device. */
+int sv_small_session_shared_bytes(sv_dtype dtype);
 /* Plans and publishes n_requests requests (host arrays as sv_run_batch_small);
  * tickets[b] identifies request b.  SV_ERR_OOM when the session holds
  * `capacity` requests in flight or its program arena is full: poll, then

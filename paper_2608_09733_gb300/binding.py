@@ -39,7 +39,8 @@ EXPORTS = ["sv_version", "sv_last_error", "sv_init_basis", "sv_apply_circuit", "
            "sv_release_scratch", "sv_profile_enable", "sv_profile_read", "sv_adjoint_grad", "sv_run_batch_small",
            "sv_expect_z_all_noalloc", "sv_emulate_apply", "sv_probabilities", "sv_sample", "sv_adjoint_grad_rows",
            "sv_batch_expect_z", "sv_adjoint_grad_ex", "sv_adjoint_grad_device", "sv_batch_expect_z_device",
-           "sv_small_session_start", "sv_small_session_submit", "sv_small_session_poll", "sv_small_session_stop",
+           "sv_small_session_start", "sv_small_session_shared_bytes", "sv_small_session_submit",
+           "sv_small_session_poll", "sv_small_session_stop",
            "sv_jit_set_mode", "sv_jit_info", "sv_jit_check", "sv_jit_check_adjoint"]
 
 
@@ -132,6 +133,7 @@ def load():
                                        ci),
             "sv_batch_expect_z_device": ([ci, ci, P(SvGate), sz, vp, ci, ci, vp, vp], ci),
             "sv_small_session_start": ([ci, ci, ci, cd, ci, P(vp)], ci),
+            "sv_small_session_shared_bytes": ([ci], ci),
             "sv_small_session_submit": ([vp, ci, P(ci), P(P(SvGate)), P(sz), P(ctypes.c_int64)], ci),
             "sv_small_session_poll": ([vp, ctypes.c_int64, P(cd), P(ci)], ci),
             "sv_small_session_stop": ([vp], ci),

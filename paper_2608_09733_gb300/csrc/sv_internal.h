@@ -172,6 +172,10 @@ template <typename R>
 cudaError_t launch_small_batch(const char* buf, const uint64_t* offset, const int* first_prog, const int* nq, int n_requests,
                                int max_n, double* out, cudaStream_t stream);
 
+// Dynamic shared memory of a session's CTA, whose largest state has max_n
+// qubits: that state.
+constexpr size_t small_session_smem(size_t amp_bytes, int max_n) { return amp_bytes << max_n; }
+
 // Persistent packed small states (serving sessions, sv_serve.cpp).  The
 // entries, published count, exit flag, results and done words are pinned host
 // memory mapped into the device; head and status are device memory.

@@ -74,6 +74,8 @@ namespace {
 std::mutex g_sessions_mu;
 std::vector<sv_small_session*> g_sessions;
 
+int session_max_n(sv_dtype d) { return d == SV_C64 ? SV_SESSION_MAX_QUBITS : 12; }
+
 size_t prog_bytes(sv_dtype d) { return d == SV_C64 ? sizeof(SweepProgram<float>) : sizeof(SweepProgram<double>); }
 
 long long load_acquire(const long long* p) {
@@ -266,7 +268,7 @@ extern "C" sv_status sv_small_session_start(sv_dtype dtype, int capacity, int ar
     if (!(wait_limit_s > 0.0 && wait_limit_s <= 3600.0)) fail(SV_ERR_INVALID, "wait_limit_s must be in (0, 3600]");
     std::unique_ptr<sv_small_session, void (*)(sv_small_session*)> s(new sv_small_session(), free_session);
     s->dtype = dtype;
-    s->max_n = dtype == SV_C64 ? SV_SESSION_MAX_QUBITS : 12;
+    s->max_n = session_max_n(dtype);
     s->capacity = capacity;
     s->arena_programs = arena_programs;
     s->limit_s = wait_limit_s;
@@ -326,6 +328,11 @@ extern "C" sv_status sv_small_session_start(sv_dtype dtype, int capacity, int ar
     }
     *out = s.release();
   });
+}
+
+extern "C" int sv_small_session_shared_bytes(sv_dtype dtype) {
+  if (dtype != SV_C64 && dtype != SV_C128) return 0;
+  return (int)small_session_smem(dtype == SV_C64 ? sizeof(Cx<float>) : sizeof(Cx<double>), session_max_n(dtype));
 }
 
 extern "C" sv_status sv_small_session_submit(sv_small_session* s, int n_requests, const int* n_qubits,

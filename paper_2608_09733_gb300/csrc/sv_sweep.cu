@@ -479,21 +479,42 @@ __global__ void __launch_bounds__(256) k_small_batch(const char* __restrict__ bu
 // (system-scope fence between them).  The wait is bounded by `limit_ns` of
 // %globaltimer: when it runs out the CTA records SV_ERR_TIMEOUT in *status
 // and returns (an idle session ends this way too).
+//
+// The CTA's shared memory is the largest state's and no more
+// (small_session_smem), so that the other kernels still fit beside a resident
+// session.  A request whose state leaves room for a program there has its
+// programs staged; a largest-size one runs them in place, from global memory:
+// plain loads, which the wait's acquire and the barrier after it order after
+// the upload, so `progs` is not __restrict__ (read-only cache loads would not
+// be).
+template <typename R, int RQ>
+__device__ __forceinline__ void run_program(const SweepProgram<R>& P, Cx<R>* s, int tsz, const Grp& gr) {
+  run_phases<R, 5, RQ, kOpsAll>(P, P.coef, s, tsz, 0ull, gr);
+}
 template <typename R>
 __device__ __forceinline__ void run_small_request(const SweepProgram<R>* progs, int first, int last, int n,
                                                   Cx<R>* s, double* red, double& result) {
   const int tsz = 1 << n;
+  uint32_t smem;
+  asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(smem));
+  const bool room = ((uint32_t)sizeof(Cx<R>) << n) + (uint32_t)staged_bytes<R>(SweepProgram<R>::kPool) <= smem;
   for (int a = threadIdx.x; a < tsz; a += blockDim.x) s[phys<R>(a)] = Cx<R>{R(a == 0 ? 1 : 0), R(0)};
   __syncthreads();
   const Grp gr{threadIdx.x, blockDim.x, 0u};
   for (int p = first; p < last; p++) {
     __syncthreads();  // the program before has been run by every thread
-    const SweepProgram<R>& P = stage_program<true>(progs[p], s + tsz);
-    __syncthreads();
-    if (P.h.rq == 5) {
-      if constexpr (sizeof(R) == 4) run_phases<R, 5, 5, kOpsAll>(P, P.coef, s, tsz, 0ull, gr);
+    if (room) {
+      const SweepProgram<R>& P = stage_program<true>(progs[p], s + tsz);
+      __syncthreads();
+      if (P.h.rq == 5) {
+        if constexpr (sizeof(R) == 4) run_program<R, 5>(P, s, tsz, gr);
+      } else {
+        run_program<R, kRegQ>(P, s, tsz, gr);
+      }
+    } else if (progs[p].h.rq == 5) {
+      if constexpr (sizeof(R) == 4) run_program<R, 5>(progs[p], s, tsz, gr);
     } else {
-      run_phases<R, 5, kRegQ, kOpsAll>(P, P.coef, s, tsz, 0ull, gr);
+      run_program<R, kRegQ>(progs[p], s, tsz, gr);
     }
   }
   // the sum runs over the first kRedThreads threads in a fixed order, so a
@@ -521,7 +542,7 @@ __device__ __forceinline__ void run_small_request(const SweepProgram<R>* progs, 
 // covers states up to 13 qubits), or 512 for sessions that take 14-qubit
 // complex64 requests (2^9 groups of 32; 128 KiB of shared memory).
 template <typename R, int NT>
-__global__ void __launch_bounds__(NT) k_small_session(SmallSessionDev d, const SweepProgram<R>* __restrict__ progs) {
+__global__ void __launch_bounds__(NT) k_small_session(SmallSessionDev d, const SweepProgram<R>* progs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cx<R>* s = reinterpret_cast<Cx<R>*>(smem_raw);
   __shared__ double red[NT / 32];
@@ -929,7 +950,7 @@ cudaError_t launch_small_session_nt(const SmallSessionDev& d, const SweepProgram
 template <typename R>
 cudaError_t launch_small_session(const SmallSessionDev& d, const SweepProgram<R>* progs, int max_n, int grid,
                                  cudaStream_t stream) {
-  const int smem = ((int)sizeof(Cx<R>) << max_n) + staged_bytes<R>(SweepProgram<R>::kPool);  // state and program
+  const int smem = (int)small_session_smem(sizeof(Cx<R>), max_n);
   if constexpr (sizeof(R) == 4)
     if (max_n >= 14) return launch_small_session_nt<R, 512>(d, progs, smem, grid, stream);
   return launch_small_session_nt<R, 256>(d, progs, smem, grid, stream);
