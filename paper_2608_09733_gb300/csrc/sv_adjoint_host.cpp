@@ -36,7 +36,7 @@ bool rotation_is_diagonal(int t) { return t == SV_GATE_RZ || t == SV_GATE_P || t
 
 // Generator G of U = exp(-i theta G / 2) on the targets: dense d x d, or the
 // d diagonal entries for the diagonal families.
-std::vector<cplx> generator_of(int t) {
+Coefs generator_of(int t) {
   const cplx j(0.0, 1.0);
   switch (t) {
     case SV_GATE_RX: return {0.0, 1.0, 1.0, 0.0};
@@ -45,18 +45,18 @@ std::vector<cplx> generator_of(int t) {
     case SV_GATE_P: return {0.0, -2.0};  // diag(1, e^{i t}) = exp(-i t (Z - I) / 2)
     case SV_GATE_RZZ: return {1.0, -1.0, -1.0, 1.0};
     case SV_GATE_RXX: {
-      std::vector<cplx> m(16, 0.0);
+      Coefs m(16, 0.0);
       m[0 * 4 + 3] = m[1 * 4 + 2] = m[2 * 4 + 1] = m[3 * 4 + 0] = 1.0;
       return m;
     }
     case SV_GATE_RYY: {
-      std::vector<cplx> m(16, 0.0);
+      Coefs m(16, 0.0);
       m[0 * 4 + 3] = m[3 * 4 + 0] = -1.0;
       m[1 * 4 + 2] = m[2 * 4 + 1] = 1.0;
       return m;
     }
     case SV_GATE_EXC1: {  // Y on the pair (|10>, |01>) = indices (1, 2)
-      std::vector<cplx> m(16, 0.0);
+      Coefs m(16, 0.0);
       m[1 * 4 + 2] = -j;
       m[2 * 4 + 1] = j;
       return m;
@@ -70,7 +70,7 @@ struct AGate {
   bool param = false;
   int slot = -1;
   int pidx = -1;        // index among the parameterised gates
-  std::vector<cplx> gen;
+  Coefs gen;
   sv_gate rec;          // the record its matrix is built from
 };
 
@@ -209,12 +209,14 @@ AdjTemplate lower_template(const sv_gate* gates, size_t ng) {
 // whose range holds that place.  A diagonal alone stays where it was.  (20
 // qubits, 10 layers of RY and RZ, 64 states: reverse passes 4.1 instead of 4.6
 // ms a segment of two layers, forward passes 1.93 instead of 2.2.)
-void group_diagonals(const std::vector<BOp>& ops, std::vector<BOp>& out) {
-  const int n = (int)ops.size();
+// Writes the grouped ops of ops[0..n) to out (room for 3 n / 2) and returns
+// their number.
+int group_diagonals(const BOp* ops, int n, BOp* out) {
   struct Range {
     int op, first, last;  // places: before op `first` .. before op `last`
   };
-  std::vector<Range> cand;
+  Range cand[kBatchOps];
+  int nc = 0;
   auto targets = [&](int j, int q) {
     if (ops[j].kind == OPK_DIAG) return false;
     for (int i = 0; i < ops[j].k; i++)
@@ -229,35 +231,43 @@ void group_diagonals(const std::vector<BOp>& ops, std::vector<BOp>& out) {
       if (targets(j, z.gq[0])) r.first = j + 1;
     for (int j = i + 1; j < n && r.last == n; j++)
       if (targets(j, z.gq[0])) r.last = j;
-    cand.push_back(r);
+    int at = nc++;  // by last place, in op order
+    for (; at > 0 && cand[at - 1].last > r.last; at--) cand[at] = cand[at - 1];
+    cand[at] = r;
   }
-  std::stable_sort(cand.begin(), cand.end(), [](const Range& a, const Range& b) { return a.last < b.last; });
-  std::vector<char> in_group(n, 0), used(cand.size(), 0);
-  std::vector<std::vector<int>> at(n + 1);  // the members of the group placed before each op
-  for (size_t a = 0; a < cand.size(); a++) {
-    if (used[a]) continue;
-    std::vector<int> m;
-    for (size_t b = a; b < cand.size(); b++)
-      if (!used[b] && cand[b].first <= cand[a].last) m.push_back((int)b);
-    if (m.size() < 2 || !at[cand[a].last].empty()) continue;
-    for (int b : m) {
-      used[b] = 1;
-      in_group[cand[b].op] = 1;
-      at[cand[a].last].push_back(cand[b].op);
-    }
+  int place[kBatchOps];  // per candidate: the op its group stands before, -1: in no group
+  char in_group[kBatchOps] = {}, taken[kBatchOps + 1] = {};
+  std::fill_n(place, nc, -1);
+  for (int a = 0; a < nc; a++) {
+    const int here = cand[a].last;
+    if (place[a] >= 0 || taken[here]) continue;
+    auto meets = [&](int b) { return place[b] < 0 && cand[b].first <= here; };
+    int m = 0;
+    for (int b = a; b < nc; b++) m += meets(b);
+    if (m < 2) continue;
+    for (int b = a; b < nc; b++)
+      if (meets(b)) {
+        place[b] = here;
+        in_group[cand[b].op] = 1;
+      }
+    taken[here] = 1;
   }
+  int no = 0;
   for (int i = 0; i <= n; i++) {
-    if (!at[i].empty()) {
-      BOp g;
+    if (taken[i]) {
+      BOp& g = out[no++];
       std::memset(&g, 0, sizeof(g));
       g.kind = OPK_ZGROUP;
-      g.k = (uint8_t)at[i].size();
-      for (int o : at[i]) g.grad |= ops[o].grad;
-      out.push_back(g);
-      for (int o : at[i]) out.push_back(ops[o]);
+      for (int b = 0; b < nc; b++) {
+        if (place[b] != i) continue;
+        g.k++;
+        g.grad |= ops[cand[b].op].grad;
+        out[no++] = ops[cand[b].op];
+      }
     }
-    if (i < n && !in_group[i]) out.push_back(ops[i]);
+    if (i < n && !in_group[i]) out[no++] = ops[i];
   }
+  return no;
 }
 
 template <typename R>
@@ -276,7 +286,7 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
     loc[sw.tq[i]] = i;
   }
   int pool = 0, nacc = 0;
-  auto put = [&](const std::vector<cplx>& v) {
+  auto put = [&](const Coefs& v) {
     int at = pool;
     for (const cplx& c : v) {
       if (pool >= BatchProgram<R>::kPool) fail(SV_ERR_INVALID, "internal: batch program pool overflow");
@@ -348,11 +358,11 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
       d.flags |= OPF_FLIP;
     if (g.param) {
       // RY has real matrices; RX, RY, RZ have Pauli generators
-      const std::vector<cplx>& G = g.gen;
+      const Coefs& G = g.gen;
       const cplx j(0.0, 1.0);
-      if (op.k == 1 && op.kind == OPK_DENSE && G == std::vector<cplx>{0.0, -j, j, 0.0}) d.flags |= OPF_REALM | OPF_GY;
-      if (op.k == 1 && op.kind == OPK_DENSE && G == std::vector<cplx>{0.0, 1.0, 1.0, 0.0}) d.flags |= OPF_GX;
-      if (op.k == 1 && op.kind == OPK_DIAG && G == std::vector<cplx>{1.0, -1.0}) d.flags |= OPF_GZ;
+      if (op.k == 1 && op.kind == OPK_DENSE && G == Coefs{0.0, -j, j, 0.0}) d.flags |= OPF_REALM | OPF_GY;
+      if (op.k == 1 && op.kind == OPK_DENSE && G == Coefs{0.0, 1.0, 1.0, 0.0}) d.flags |= OPF_GX;
+      if (op.k == 1 && op.kind == OPK_DIAG && G == Coefs{1.0, -1.0}) d.flags |= OPF_GZ;
       d.table = 1;
       d.coef = (uint32_t)g.pidx;
       if (reverse) {
@@ -401,8 +411,8 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
       BOp& d = P.ops[o];
       for (int i = 0; i < d.k; i++)
         d.rs[i] = (d.pos[i] != 0xFF && slot_of[d.pos[i]] >= 0) ? (uint8_t)slot_of[d.pos[i]] : 0xFF;
-      for (int q = 0; q < sw.m; q++) {
-        if (!((d.lmask >> q) & 1u)) continue;
+      for (uint32_t lm = d.lmask; lm; lm &= lm - 1) {
+        const int q = __builtin_ctz(lm);
         const bool v = (d.lval >> q) & 1u;
         if (slot_of[q] >= 0) {
           d.rmask |= 1u << slot_of[q];
@@ -435,21 +445,21 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
   P.h.nphases = nph;
 
   // one-qubit diagonals of a register phase in groups (OPK_ZGROUP)
-  std::vector<BOp> fin;
+  BOp fin[kBatchOps + kBatchOps / 2];
+  int nfin = 0;
   for (int p = 0; p < nph; p++) {
     Phase& ph = P.ph[p];
-    const std::vector<BOp> list(P.ops + ph.first, P.ops + ph.first + ph.nops);
-    const size_t at = fin.size();
+    const int at = nfin;
     if (ph.kind == PH_REG)
-      group_diagonals(list, fin);
+      nfin += group_diagonals(P.ops + ph.first, ph.nops, fin + at);
     else
-      fin.insert(fin.end(), list.begin(), list.end());
+      nfin = (int)(std::copy_n(P.ops + ph.first, ph.nops, fin + at) - fin);
     ph.first = (uint8_t)at;
-    ph.nops = (uint8_t)(fin.size() - at);
+    ph.nops = (uint8_t)(nfin - at);
   }
-  if ((int)fin.size() > kBatchOps) fail(SV_ERR_INVALID, "internal: too many ops in a batch program");
-  std::copy(fin.begin(), fin.end(), P.ops);
-  P.h.nops = (int)fin.size();
+  if (nfin > kBatchOps) fail(SV_ERR_INVALID, "internal: too many ops in a batch program");
+  std::copy_n(fin, nfin, P.ops);
+  P.h.nops = nfin;
   P.h.ngacc = nacc;
   // offsets of each op's matrix and generator in the CTA's shared copy, and of
   // each group's table (16-byte aligned)
@@ -479,18 +489,14 @@ template <typename R, typename F>
 void segment_programs(const AdjTemplate& T, size_t g0, size_t g1, bool reverse, int n, int batch, int tile_q,
                       int low_q, BatchProgram<R>& prog, F&& each) {
   std::vector<int> order;
-  std::vector<LOp> ops;
-  if (!reverse) {
-    for (size_t i = T.start[g0]; i < T.start[g1]; i++) {
-      order.push_back((int)i);
-      ops.push_back(T.ag[i].op);
-    }
-  } else {
-    for (size_t i = T.start[g1]; i-- > T.start[g0];) {
-      order.push_back((int)i);
-      ops.push_back(T.ag[i].op);
-    }
-  }
+  std::vector<const LOp*> ops;
+  order.reserve(T.start[g1] - T.start[g0]);
+  ops.reserve(T.start[g1] - T.start[g0]);
+  if (!reverse)
+    for (size_t i = T.start[g0]; i < T.start[g1]; i++) order.push_back((int)i);
+  else
+    for (size_t i = T.start[g1]; i-- > T.start[g0];) order.push_back((int)i);
+  for (int i : order) ops.push_back(&T.ag[i].op);
   std::vector<Sweep> sws = schedule_sweeps(n, ops, tile_q, low_q, BatchProgram<R>::kPool / 2, 64, true);
   for (const Sweep& sw : sws) {
     fill_program<R>(T.ag, order, sw, n, batch, T.npg, reverse, prog);
@@ -601,7 +607,7 @@ void run_adjoint(int n, sv_dtype dtype, const sv_gate* gates, size_t ng, const d
     pslot.push_back(ag[i].slot);
     if (dev) continue;
     for (int b = 0; b < batch; b++) {
-      std::vector<cplx> U = gate_matrix(ag[i].rec, params + (size_t)b * npar);
+      Coefs U = gate_matrix(ag[i].rec, params + (size_t)b * npar);
       Cx<R>* row = &table[((size_t)ag[i].pidx * batch + b) * kTableStride];
       int d = 1 << ag[i].rec.n_targets;
       if (ag[i].op.kind == OPK_DIAG)

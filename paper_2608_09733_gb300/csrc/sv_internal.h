@@ -5,7 +5,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <complex>
+#include <initializer_list>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -18,15 +21,78 @@ using cplx = std::complex<double>;
 
 // ----------------------------------------------------------------- host plan
 
+// The coefficients of one operation: a vector whose first four entries (a
+// one-qubit matrix, a two-qubit diagonal) need no allocation.  A plan copies
+// its operations a few times, and most of them are that small.
+class Coefs {
+ public:
+  Coefs() = default;
+  Coefs(std::initializer_list<cplx> l) { assign(l.begin(), l.end()); }
+  Coefs(size_t n, cplx v) { assign(n, v); }
+  Coefs(const Coefs& o) { assign(o.begin(), o.end()); }
+  Coefs(Coefs&& o) noexcept { take(o); }
+  Coefs& operator=(const Coefs& o) {
+    if (this != &o) assign(o.begin(), o.end());
+    return *this;
+  }
+  Coefs& operator=(Coefs&& o) noexcept {
+    if (this != &o) take(o);
+    return *this;
+  }
+  // [b, e) must not point into this object
+  void assign(const cplx* b, const cplx* e) { std::copy(b, e, room((size_t)(e - b))); }
+  void assign(size_t n, cplx v) { std::fill_n(room(n), n, v); }
+  void clear() { n_ = 0; }
+  size_t size() const { return n_; }
+  cplx* data() { return at_; }
+  const cplx* data() const { return at_; }
+  cplx* begin() { return at_; }
+  cplx* end() { return at_ + n_; }
+  const cplx* begin() const { return at_; }
+  const cplx* end() const { return at_ + n_; }
+  cplx& operator[](size_t i) { return at_[i]; }
+  const cplx& operator[](size_t i) const { return at_[i]; }
+  bool operator==(const Coefs& o) const { return n_ == o.n_ && std::equal(begin(), end(), o.begin()); }
+
+ private:
+  static constexpr size_t kSmall = 4;
+  cplx* room(size_t n) {
+    if (n > cap_) {
+      big_.reset(new cplx[n]);
+      at_ = big_.get();
+      cap_ = n;
+    }
+    n_ = n;
+    return at_;
+  }
+  void take(Coefs& o) {
+    if (o.big_) {
+      big_ = std::move(o.big_);
+      at_ = big_.get();
+      cap_ = o.cap_;
+      n_ = o.n_;
+      o.at_ = o.small_;
+      o.cap_ = kSmall;
+    } else {
+      assign(o.begin(), o.end());
+    }
+    o.n_ = 0;
+  }
+  size_t n_ = 0, cap_ = kSmall;
+  cplx* at_ = small_;
+  cplx small_[kSmall];
+  std::unique_ptr<cplx[]> big_;
+};
+
 // A gate after lowering (a matrix in double precision) or a fused block.
 struct LOp {
   OpKind kind = OPK_DENSE;
-  int k = 0;                 // matrix qubits
-  int q[5] = {0, 0, 0, 0, 0};  // global matrix qubits, q[0] = least significant matrix bit
-  int nc = 0;
-  int c[5] = {0, 0, 0, 0, 0};  // global control qubits
-  int cs[5] = {1, 1, 1, 1, 1}; // required control states
-  std::vector<cplx> m;       // DENSE/REAL: 2^k x 2^k row-major; DIAG: 2^k; ANTIDIAG: {a, b}
+  int8_t k = 0;                   // matrix qubits
+  int8_t q[5] = {0, 0, 0, 0, 0};  // global matrix qubits, q[0] = least significant matrix bit
+  int8_t nc = 0;
+  int8_t c[5] = {0, 0, 0, 0, 0};   // global control qubits
+  int8_t cs[5] = {1, 1, 1, 1, 1};  // required control states
+  Coefs m;                   // DENSE/REAL: 2^k x 2^k row-major; DIAG: 2^k; ANTIDIAG: {a, b}
   uint64_t touch = 0;        // every qubit the op reads (matrix qubits and controls)
   uint64_t need = 0;         // qubits that must be inside the tile
   int first_gate = 0;        // index of the first source gate (fusion bookkeeping)
@@ -99,12 +165,12 @@ Pinned& pinned_buffer(cudaStream_t stream, const char* name, size_t bytes);
 // Lowering (gate records -> double-precision matrices), the paper's greedy
 // fusion, and the tile scheduler.  Throw sv::Error on invalid input.
 void validate_gates(int n, const sv_gate* gates, size_t n_gates, size_t n_param_values);
-std::vector<cplx> gate_matrix(const sv_gate& g, const double* param_values);
+Coefs gate_matrix(const sv_gate& g, const double* param_values);
 LOp lower_gate(const sv_gate& g, const double* param_values, int index);
 std::vector<LOp> fuse_greedy(int n, const sv_gate* gates, size_t n_gates, const double* param_values, int kmax,
                              std::vector<int>* block_starts, bool dense_always);
 void classify(LOp& op);
-std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_q, int low_q, int coef_pool,
+std::vector<Sweep> schedule_sweeps(int n, const std::vector<const LOp*>& ops, int tile_q, int low_q, int coef_pool,
                                    int ops_per_pass, bool commute);
 Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, const double* param_values,
                size_t n_param_values, const sv_exec_opts& opts, int tile_q_override = 0, bool lane = false);

@@ -77,31 +77,31 @@ void validate_gates(int n, const sv_gate* gates, size_t n_gates, size_t n_param_
   if (n_gates && !gates) fail(SV_ERR_INVALID, "gates is NULL");
   for (size_t gi = 0; gi < n_gates; gi++) {
     const sv_gate& g = gates[gi];
-    std::string at = "gate " + std::to_string(gi) + ": ";
-    if (g.type < 0 || g.type >= SV_GATE_COUNT_) fail(SV_ERR_INVALID, at + "unknown gate type");
+    auto at = [&] { return "gate " + std::to_string(gi) + ": "; };  // the text of an error only
+    if (g.type < 0 || g.type >= SV_GATE_COUNT_) fail(SV_ERR_INVALID, at() + "unknown gate type");
     int want = kTargetsOf[g.type];
-    if (want > 0 && g.n_targets != want) fail(SV_ERR_INVALID, at + "wrong number of targets for its family");
-    if (g.n_targets < 1 || g.n_targets > SV_MAX_TARGETS) fail(SV_ERR_INVALID, at + "n_targets out of range");
-    if (g.n_controls < 0 || g.n_controls > SV_MAX_CONTROLS) fail(SV_ERR_INVALID, at + "n_controls out of range");
+    if (want > 0 && g.n_targets != want) fail(SV_ERR_INVALID, at() + "wrong number of targets for its family");
+    if (g.n_targets < 1 || g.n_targets > SV_MAX_TARGETS) fail(SV_ERR_INVALID, at() + "n_targets out of range");
+    if (g.n_controls < 0 || g.n_controls > SV_MAX_CONTROLS) fail(SV_ERR_INVALID, at() + "n_controls out of range");
     uint64_t seen = 0;
     for (int i = 0; i < g.n_targets + g.n_controls; i++) {
       int q = i < g.n_targets ? g.targets[i] : g.controls[i - g.n_targets];
-      if (q < 0 || q >= n) fail(SV_ERR_INVALID, at + "qubit " + std::to_string(q) + " out of range");
-      if (seen & (1ull << q)) fail(SV_ERR_INVALID, at + "qubit " + std::to_string(q) + " repeated");
+      if (q < 0 || q >= n) fail(SV_ERR_INVALID, at() + "qubit " + std::to_string(q) + " out of range");
+      if (seen & (1ull << q)) fail(SV_ERR_INVALID, at() + "qubit " + std::to_string(q) + " repeated");
       seen |= 1ull << q;
     }
     if (g.n_controls < 32 && (g.control_zero_mask >> g.n_controls) != 0)
-      fail(SV_ERR_INVALID, at + "control_zero_mask has bits beyond n_controls");
+      fail(SV_ERR_INVALID, at() + "control_zero_mask has bits beyond n_controls");
     for (int i = 0; i < kAnglesOf[g.type]; i++) {
       int s = g.param_slot[i];
-      if (s < -1) fail(SV_ERR_INVALID, at + "negative parameter slot");
+      if (s < -1) fail(SV_ERR_INVALID, at() + "negative parameter slot");
       if (s >= 0 && (size_t)s >= n_param_values)
-        fail(SV_ERR_UNBOUND_PARAM, at + "parameter slot " + std::to_string(s) + " is unbound");
+        fail(SV_ERR_UNBOUND_PARAM, at() + "parameter slot " + std::to_string(s) + " is unbound");
       double v = s >= 0 ? 0.0 : g.params[i];
-      if (!std::isfinite(v)) fail(SV_ERR_INVALID, at + "angle is not finite");
+      if (!std::isfinite(v)) fail(SV_ERR_INVALID, at() + "angle is not finite");
     }
     if (g.type == SV_GATE_UNITARY) {
-      if (!g.matrix) fail(SV_ERR_INVALID, at + "unitary gate without a matrix");
+      if (!g.matrix) fail(SV_ERR_INVALID, at() + "unitary gate without a matrix");
       int d = 1 << g.n_targets;
       // U^dagger U = I within 1e-6 (a user matrix that is not unitary is rejected)
       double worst = 0.0;
@@ -115,14 +115,14 @@ void validate_gates(int n, const sv_gate* gates, size_t n_gates, size_t n_param_
           }
           worst = std::max(worst, std::abs(acc - (r == c ? 1.0 : 0.0)));
         }
-      if (!(worst < 1e-6)) fail(SV_ERR_INVALID, at + "matrix is not unitary");
+      if (!(worst < 1e-6)) fail(SV_ERR_INVALID, at() + "matrix is not unitary");
     }
   }
 }
 
 // The matrix of a gate (without its controls), from the definitions of the
 // gate table (Sec. 4.2) and R_P(theta) = exp(-i theta P / 2) (Sec. 9.1).
-std::vector<cplx> gate_matrix(const sv_gate& g, const double* pv) {
+Coefs gate_matrix(const sv_gate& g, const double* pv) {
   auto ang = [&](int i) { return g.param_slot[i] >= 0 ? pv[g.param_slot[i]] : g.params[i]; };
   const cplx j(0.0, 1.0);
   const double h = 1.0 / std::sqrt(2.0);
@@ -156,7 +156,7 @@ std::vector<cplx> gate_matrix(const sv_gate& g, const double* pv) {
       return {c, -std::polar(s, la), std::polar(s, ph), std::polar(c, ph + la)};
     }
     case SV_GATE_SWAP: {
-      std::vector<cplx> m(16, 0.0);
+      Coefs m(16, 0.0);
       m[0] = m[15] = 1.0;
       m[1 * 4 + 2] = m[2 * 4 + 1] = 1.0;
       return m;
@@ -167,7 +167,7 @@ std::vector<cplx> gate_matrix(const sv_gate& g, const double* pv) {
       // -1 on its outer anti-diagonal corners and +1 on the inner ones.
       double c = std::cos(0.5 * ang(0)), s = std::sin(0.5 * ang(0));
       double outer = g.type == SV_GATE_RXX ? 1.0 : -1.0;
-      std::vector<cplx> m(16, 0.0);
+      Coefs m(16, 0.0);
       for (int r = 0; r < 4; r++) m[r * 4 + r] = c;
       m[0 * 4 + 3] = m[3 * 4 + 0] = -j * s * outer;
       m[1 * 4 + 2] = m[2 * 4 + 1] = -j * s;
@@ -176,13 +176,13 @@ std::vector<cplx> gate_matrix(const sv_gate& g, const double* pv) {
     case SV_GATE_RZZ: {
       // Z(x)Z = diag(1, -1, -1, 1)
       cplx a = std::polar(1.0, -0.5 * ang(0)), b = std::polar(1.0, 0.5 * ang(0));
-      std::vector<cplx> m(16, 0.0);
+      Coefs m(16, 0.0);
       m[0] = a; m[5] = b; m[10] = b; m[15] = a;
       return m;
     }
     case SV_GATE_UNITARY: {
       int d = 1 << g.n_targets;
-      std::vector<cplx> m(d * d);
+      Coefs m(d * d, 0.0);
       for (int i = 0; i < d * d; i++) m[i] = cplx(g.matrix[2 * i], g.matrix[2 * i + 1]);
       return m;
     }
@@ -193,7 +193,7 @@ std::vector<cplx> gate_matrix(const sv_gate& g, const double* pv) {
       const int d = g.type == SV_GATE_EXC1 ? 4 : 16, a = g.type == SV_GATE_EXC1 ? 1 : 3,
                 b = g.type == SV_GATE_EXC1 ? 2 : 12;
       const double c = std::cos(0.5 * ang(0)), s = std::sin(0.5 * ang(0));
-      std::vector<cplx> m(d * d, 0.0);
+      Coefs m(d * d, 0.0);
       for (int r = 0; r < d; r++) m[r * d + r] = 1.0;
       m[a * d + a] = c;
       m[a * d + b] = -s;
@@ -207,7 +207,7 @@ std::vector<cplx> gate_matrix(const sv_gate& g, const double* pv) {
 
 void classify(LOp& op) {
   const int d = 1 << op.k;
-  const std::vector<cplx>& m = op.m;
+  const Coefs& m = op.m;
   op.touch = 0;
   for (int i = 0; i < op.k; i++) op.touch |= 1ull << op.q[i];
   for (int i = 0; i < op.nc; i++) op.touch |= 1ull << op.c[i];
@@ -222,10 +222,10 @@ void classify(LOp& op) {
       if (v.imag() != 0.0) real = false;
     }
   if (diag) {
-    std::vector<cplx> dd(d);
+    Coefs dd(d, 0.0);
     for (int r = 0; r < d; r++) dd[r] = m[r * d + r];
     op.kind = OPK_DIAG;
-    op.m = dd;
+    op.m = std::move(dd);
     op.need = 0;  // a diagonal never moves amplitudes: any tile can apply it
     return;
   }
@@ -270,7 +270,7 @@ LOp lower_gate(const sv_gate& g, const double* pv, int index) {
 
 // Applies gate g, re-indexed onto the block's local qubits, to a vector of
 // 2^nb amplitudes (used to build a fused block's matrix column by column).
-static void apply_local(std::vector<cplx>& v, int nb, const sv_gate& g, const std::vector<cplx>& U,
+static void apply_local(std::vector<cplx>& v, int nb, const sv_gate& g, const Coefs& U,
                         const int* local_of) {
   int k = g.n_targets, d = 1 << k;
   int t[5];
@@ -378,7 +378,7 @@ std::vector<LOp> fuse_greedy(int n, const sv_gate* gates, size_t n_gates, const 
     op.k = nb;
     int d = 1 << nb;
     op.m.assign((size_t)d * d, 0.0);
-    std::vector<std::vector<cplx>> mats;
+    std::vector<Coefs> mats;
     for (size_t g = start; g < i; g++) mats.push_back(gate_matrix(gates[g], pv));
     std::vector<std::vector<cplx>> cols((size_t)d, std::vector<cplx>((size_t)d, cplx(0.0)));
     for (int c = 0; c < d; c++) cols[c][c] = 1.0;
@@ -421,7 +421,7 @@ PhaseOp phase_op(const LOp& op, uint32_t need, bool smem) {
 // shares with them both act diagonally (controls and diagonals commute), not
 // only when it shares none: CZ layers then hold up fewer ops (20 layers of U3
 // and CZ on 30 qubits: 35 passes against 38, on 24 qubits 25 against 28).
-std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_q, int low_q, int coef_pool,
+std::vector<Sweep> schedule_sweeps(int n, const std::vector<const LOp*>& ops, int tile_q, int low_q, int coef_pool,
                                    int ops_per_pass, bool commute) {
   const int max_ops = ops_per_pass > 0 ? std::min(ops_per_pass, kMaxOps) : kMaxOps;
   std::vector<Sweep> out;
@@ -437,7 +437,7 @@ std::vector<Sweep> schedule_sweeps(int n, const std::vector<LOp>& ops, int tile_
     int coef = 0;
     for (size_t i = first; i < ops.size(); i++) {
       if (done[i]) continue;
-      const LOp& op = ops[i];
+      const LOp& op = *ops[i];
       PhaseOp p = phase_op(op, 0, false);
       if (!commute) p = {op.touch, 0, 0, false};
       const bool blocked = (p.moves & (moved | held)) || (p.holds & moved);
@@ -517,7 +517,7 @@ std::vector<int> order_by_phase(const std::vector<PhaseOp>& ops, int rq, int* ph
 // table of the next gate on the same qubit, possibly in a later pass, instead
 // of costing a phase table of its own.  Ops the factors do not reproduce
 // within tol stay whole.
-static void split_one_qubit(std::vector<LOp>& ops, double tol) {
+static std::vector<LOp> split_one_qubit(const std::vector<LOp>& ops, double tol) {
   // Worth it only where the closing diagonal has a table to join: the next
   // op that targets the qubit (diagonals aside) is another uncontrolled
   // one-qubit gate.  Before a CNOT target, say, it would cost a table anyway.
@@ -533,10 +533,10 @@ static void split_one_qubit(std::vector<LOp>& ops, double tol) {
   std::vector<LOp> out;
   out.reserve(ops.size() * 2);
   for (size_t i = 0; i < ops.size(); i++) {
-    LOp& op = ops[i];
+    const LOp& op = ops[i];
     RotSplit r;
     if (!(split[i] && rot_split(op.m.data(), tol, r))) {
-      out.push_back(std::move(op));
+      out.push_back(op);
       continue;
     }
     auto part = [&](cplx m00, cplx m01, cplx m10, cplx m11) {
@@ -551,7 +551,7 @@ static void split_one_qubit(std::vector<LOp>& ops, double tol) {
     out.push_back(part(r.C, -r.S * r.elam, r.S, r.C * r.elam));
     out.push_back(part(r.g, 0.0, 0.0, r.g * r.ephi));
   }
-  ops = std::move(out);
+  return out;
 }
 
 // Joins one-qubit gates into the two-qubit matrices beside them: a one-qubit
@@ -586,7 +586,7 @@ static void join_one_qubit(std::vector<LOp>& ops) {
     return u;
   };
   // u on matrix bit `bit` of a two-qubit op: rows (after it) or columns (before it)
-  auto apply = [](std::vector<cplx>& m, const Mat2& u, int bit, bool after) {
+  auto apply = [](Coefs& m, const Mat2& u, int bit, bool after) {
     const int s = 1 << bit;
     for (int r = 0; r < 4; r++) {
       if (r & s) continue;
@@ -640,7 +640,7 @@ static void join_one_qubit(std::vector<LOp>& ops) {
         }
       const int l = last[op.q[0]];
       if (l >= 0 && l == last[op.q[1]] && two(out[l])) {  // the same pair again
-        std::vector<cplx> m(16, 0.0);
+        Coefs m(16, 0.0);
         const bool flip = out[l].q[0] != op.q[0];
         auto at = [&](int i) { return flip ? ((i & 1) << 1) | (i >> 1) : i; };
         for (int r = 0; r < 4; r++)
@@ -763,18 +763,12 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
   }
   // drop exact identities (e.g. the I gate): they move no amplitude
   auto drop_identities = [](std::vector<LOp>& ops) {
-    std::vector<LOp> kept;
-    kept.reserve(ops.size());
-    for (auto& op : ops) {
-      if (op.kind == OPK_DIAG) {
-        bool ident = true;
-        for (auto& v : op.m)
-          if (v != 1.0) ident = false;
-        if (ident) continue;
-      }
-      kept.push_back(std::move(op));
-    }
-    ops = std::move(kept);
+    ops.erase(std::remove_if(ops.begin(), ops.end(),
+                             [](const LOp& op) {
+                               return op.kind == OPK_DIAG &&
+                                      std::all_of(op.m.begin(), op.m.end(), [](const cplx& v) { return v == 1.0; });
+                             }),
+              ops.end());
   };
   drop_identities(p.ops);
   if (opts.ops_per_pass != 1 && opts.block_mode == SV_BLOCK_AUTO && tile_q_override == 0) {
@@ -792,24 +786,28 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
   // has more tables (20 layers of U3 and CZ on 24 qubits: 28 passes 48.3 ms,
   // 29 passes 46.3).
   const bool commute = tile_q_override == 0 && (dtype == SV_C64 || lane);
-  p.sweeps = schedule_sweeps(n, p.ops, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass, commute);
+  auto schedule = [&](const std::vector<LOp>& ops) {
+    std::vector<const LOp*> list;
+    list.reserve(ops.size());
+    for (const LOp& op : ops) list.push_back(&op);
+    return schedule_sweeps(n, list, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass, commute);
+  };
+  p.sweeps = schedule(p.ops);
   if (opts.ops_per_pass != 1) {
-    defer_diagonals(p.ops, p.sweeps, max_ops, pool);
     // The split form has more ops, which can cut the greedy passes short and
     // leave more of them: keep it only when it needs no more passes, or at most
     // one in twenty more.  Whole gates close with a table of their own in each
     // phase: 20 layers of U3 and CZ on 28 qubits take 31.8 ms with 32 passes
     // and 252 tables, 28.7 ms with 33 passes and 162.
-    std::vector<LOp> ops2 = p.ops;
-    split_one_qubit(ops2, dtype == SV_C64 ? 1e-9 : 1e-13);
+    std::vector<LOp> ops2 = split_one_qubit(p.ops, dtype == SV_C64 ? 1e-9 : 1e-13);
     drop_identities(ops2);
-    std::vector<Sweep> sw2 = schedule_sweeps(n, ops2, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass, commute);
+    std::vector<Sweep> sw2 = schedule(ops2);
     const size_t more = commute ? p.sweeps.size() / 20 : 0;
     if (sw2.size() <= p.sweeps.size() + more) {
-      defer_diagonals(ops2, sw2, max_ops, pool);
       p.ops = std::move(ops2);
       p.sweeps = std::move(sw2);
     }
+    defer_diagonals(p.ops, p.sweeps, max_ops, pool);
   }
   return p;
 }

@@ -26,31 +26,36 @@ constexpr bool g_rot_split = SV_ROT_SPLIT != 0;  // register phases in rotation 
 
 }  // namespace
 
+// a * b without the complex product's recovery of infinities: no coefficient is
+// infinite, and a table is a few hundred products.
+static inline cplx times(const cplx& a, const cplx& b) {
+  return {a.real() * b.real() - a.imag() * b.imag(), a.real() * b.imag() + a.imag() * b.real()};
+}
+
 // A 2x2 unitary U written as g * diag(1, ephi) * [[C, -S], [S, C]] * diag(1, elam)
 // with C = |U00| and S = |U10| (C^2 + S^2 = 1, |g| = |ephi| = |elam| = 1): the
 // Z-Y-Z Euler form of a one-qubit gate, C = cos(alpha), S = sin(alpha), alpha
 // in [0, pi/2].
 bool rot_split(const cplx* U, double tol, RotSplit& r) {
-  double C = std::abs(U[0]), S = std::abs(U[2]);
+  const double a0 = std::abs(U[0]), a1 = std::abs(U[1]), a2 = std::abs(U[2]), a3 = std::abs(U[3]);
+  double C = a0, S = a2;
   const double nrm = std::hypot(C, S);
   if (!(nrm > 0.5 && nrm < 2.0)) return false;
   C /= nrm;
   S /= nrm;
   constexpr double tiny = 1e-150;
-  const cplx g = std::abs(U[0]) > tiny ? U[0] / std::abs(U[0])
-                 : std::abs(U[1]) > tiny ? -U[1] / std::abs(U[1])
-                                          : cplx(1.0);
+  const cplx g = a0 > tiny ? U[0] / a0 : a1 > tiny ? -U[1] / a1 : cplx(1.0);
   cplx ephi = 1.0, elam = 1.0;
-  if (std::abs(U[2]) > tiny && std::abs(U[1]) > tiny) {
-    ephi = (U[2] / std::abs(U[2])) / g;
-    elam = -(U[1] / std::abs(U[1])) / g;
-  } else if (std::abs(U[3]) > tiny) {  // diagonal
-    ephi = (U[3] / std::abs(U[3])) / g;
+  if (a2 > tiny && a1 > tiny) {
+    ephi = (U[2] / a2) / g;
+    elam = -(U[1] / a1) / g;
+  } else if (a3 > tiny) {  // diagonal
+    ephi = (U[3] / a3) / g;
   }
   // reconstruct and compare
   const cplx M[4] = {g * C, -g * S * elam, g * ephi * S, g * ephi * elam * C};
   for (int i = 0; i < 4; i++)
-    if (!(std::abs(M[i] - U[i]) <= tol)) return false;
+    if (!(std::norm(M[i] - U[i]) <= tol * tol)) return false;
   r.g = g;
   r.ephi = ephi;
   r.elam = elam;
@@ -86,7 +91,7 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
   const bool reg_ok = sw.m >= rq && (plan.lane || sw.m - rq <= 8);
   struct Tmp {
     DevOp d;
-    std::vector<cplx> m;
+    Coefs m;
     bool smem;
     uint32_t need;  // local positions that must be register slots
   };
@@ -274,11 +279,11 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
         std::swap(d.pos[0], d.pos[1]);
         std::swap(d.gq[0], d.gq[1]);
         if (t.m.size() == 16) {
-          std::vector<cplx> mt(16);
+          Coefs mt(16, 0.0);
           auto sw2 = [](int x) { return ((x & 1) << 1) | ((x >> 1) & 1); };
           for (int r = 0; r < 4; r++)
             for (int c = 0; c < 4; c++) mt[r * 4 + c] = t.m[sw2(r) * 4 + sw2(c)];
-          t.m = mt;
+          t.m = std::move(mt);
         }
       }
     }
@@ -393,13 +398,13 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
     return t;
   };
   // Per-slot products of uncontrolled one-qubit gates, in order.
-  auto merge_ops = [&](const std::vector<int>& list, std::vector<cplx>& mats) {
+  auto merge_ops = [&](const std::vector<int>& list, Coefs& mats) {
     mats.assign(4 * rq, 0.0);
     for (int s2 = 0; s2 < rq; s2++) mats[4 * s2] = mats[4 * s2 + 3] = 1.0;
     uint32_t present = 0;
     for (int o : list) {
       const int sl = ts[o].d.rs[0];
-      const std::vector<cplx>& U = ts[o].m;
+      const Coefs& U = ts[o].m;
       cplx* M = &mats[4 * sl];
       const cplx a = U[0] * M[0] + U[1] * M[2], b = U[0] * M[1] + U[1] * M[3];
       const cplx c = U[2] * M[0] + U[3] * M[2], d = U[2] * M[1] + U[3] * M[3];
@@ -408,7 +413,7 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
     }
     return present;
   };
-  auto kron_op = [&](uint32_t present, const std::vector<cplx>& mats) {
+  auto kron_op = [&](uint32_t present, const Coefs& mats) {
     Tmp k = blank(OPK_KRON);
     k.d.rmask = (uint8_t)present;
     k.m = mats;
@@ -421,7 +426,7 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
         while (end < first + nops && u1_free(ts[end])) end++;
         std::vector<int> list;
         for (int x = o; x < end; x++) list.push_back(x);
-        std::vector<cplx> mats;
+        Coefs mats;
         const uint32_t present = merge_ops(list, mats);
         fin.push_back(kron_op(present, mats));
         o = end;
@@ -440,6 +445,13 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
     std::vector<cplx> tab(NT, 1.0);    // [variant][register combination]
     cplx sc = 1.0;
     auto nvar = [&] { return 1 << (int)sel.size(); };
+    // the entries with register slot s set times f (bit s of an entry's index is
+    // bit s of its register combination: NT = 2^rq)
+    auto scale_slot = [&](int s, cplx f) {
+      if (f == cplx(1.0)) return;
+      const int bit = 1 << s;
+      for (int x = bit; x < nvar() * NT; x = (x + 1) | bit) tab[x] = times(tab[x], f);
+    };
     auto tab_dep = [&](uint32_t slots) {
       for (int v = 0; v < nvar(); v++)
         for (int j = 0; j < NT; j++)
@@ -458,8 +470,8 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
         const int stride = table_stride<R>(rq);  // padded: variants start in different banks
         t.m.assign((size_t)nvar() * stride, 0.0);
         for (int v = 0; v < nvar(); v++)
-          for (int j = 0; j < NT; j++) t.m[v * stride + j] = tab[v * NT + j] * sc;
-        fin.push_back(t);
+          for (int j = 0; j < NT; j++) t.m[v * stride + j] = times(tab[v * NT + j], sc);
+        fin.push_back(std::move(t));
       }
       sel.clear();
       tab.assign(NT, 1.0);
@@ -500,15 +512,19 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
       const DevOp& d = t.d;
       std::vector<int> codes;
       if (!need_codes(d, codes)) return false;
-      auto sel_bit = [&](int code, int v) { return (v >> selector(code)) & 1; };
-      for (int c : codes) selector(c);  // make sure every needed selector exists
+      uint32_t vm = 0, vv = 0;  // the variants it acts on: (v & vm) == vv
+      auto control = [&](int code, bool want) {
+        vm |= 1u << selector(code);
+        if (want) vv |= 1u << selector(code);
+      };
+      for (uint32_t t2 = d.tmask; t2; t2 &= t2 - 1) control(__builtin_ctz(t2), (d.tval & t2 & (0u - t2)) != 0);
+      for (uint64_t x2 = d.xmask; x2; x2 &= x2 - 1) control(64 + __builtin_ctzll(x2), (d.xval & x2 & (0ull - x2)) != 0);
+      int mat_sel[2] = {0, 0};  // selectors of matrix bits outside the registers
+      if (d.kind == OPK_DIAG)
+        for (int i = 0; i < d.k; i++)
+          if (d.rs[i] == 0xFF) mat_sel[i] = selector(d.pos[i] != 0xFF ? (int)d.pos[i] : 64 + (int)d.gq[i]);
       for (int v = 0; v < nvar(); v++) {
-        bool on = true;
-        for (int q = 0; q < 32; q++)
-          if ((d.tmask >> q) & 1u) on = on && sel_bit(q, v) == (int)((d.tval >> q) & 1u);
-        for (int q = 0; q < 64; q++)
-          if ((d.xmask >> q) & 1ull) on = on && sel_bit(64 + q, v) == (int)((d.xval >> q) & 1ull);
-        if (!on) continue;
+        if (((uint32_t)v & vm) != vv) continue;
         for (int j = 0; j < NT; j++) {
           if (((uint32_t)j & d.rmask) != d.rval) continue;
           cplx& x = tab[v * NT + j];
@@ -516,15 +532,8 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
             x = -x;
           } else {
             int idx = 0;
-            for (int i = 0; i < d.k; i++) {
-              int b;
-              if (d.rs[i] != 0xFF)
-                b = (j >> d.rs[i]) & 1;
-              else
-                b = sel_bit(d.pos[i] != 0xFF ? (int)d.pos[i] : 64 + (int)d.gq[i], v);
-              idx |= b << i;
-            }
-            x *= t.m[idx];
+            for (int i = 0; i < d.k; i++) idx |= ((d.rs[i] != 0xFF ? j >> d.rs[i] : v >> mat_sel[i]) & 1) << i;
+            x = times(x, t.m[idx]);
           }
         }
       }
@@ -600,7 +609,7 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
         }
         for (int h : hoist)
           if (!fold_or_restart(ts[h])) fin.push_back(ts[h]);
-        std::vector<cplx> mats;
+        Coefs mats;
         const uint32_t present = merge_ops(list, mats);
         o = end;
         RotSplit sp[kMaxRegQ];
@@ -614,8 +623,7 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
         }
         for (int s2 = 0; s2 < rq; s2++) {
           if (!((present >> s2) & 1u)) continue;
-          for (int x = 0; x < nvar() * NT; x++)
-            if ((x >> s2) & 1) tab[x] *= sp[s2].elam;  // bit s2 of x is bit s2 of j (NT = 2^rq)
+          scale_slot(s2, sp[s2].elam);
           sc *= sp[s2].g;
         }
         // complex128 takes the scaled form (two multiply-adds per component),
@@ -647,12 +655,10 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
         }
         fin.push_back(k);
         for (int s2 = 0; s2 < rq; s2++) {
-          if (!((present >> s2) & 1u)) continue;
-          for (int x = 0; x < nvar() * NT; x++)
-            if ((x >> s2) & 1) tab[x] *= sp[s2].ephi;
+          if ((present >> s2) & 1u) scale_slot(s2, sp[s2].ephi);
         }
         // the scaled form lets the amplitudes grow by up to sqrt(2) per rotation
-        if (std::abs(sc) < 1e-30) flush();
+        if (std::norm(sc) < 1e-60) flush();
         continue;
       }
       if ((d.kind == OPK_SIGN || d.kind == OPK_DIAG) && fold_or_restart(t)) {
