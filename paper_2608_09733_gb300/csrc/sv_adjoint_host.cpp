@@ -200,8 +200,9 @@ AdjTemplate lower_template(const sv_gate* gates, size_t ng) {
   return T;
 }
 
-// The ops of one register phase with its uncontrolled one-qubit diagonals
-// (without a gradient, or with the Z generator) gathered into groups.  Such an
+// The ops of one register phase with its uncontrolled one-qubit diagonals of
+// modulus one (without a gradient, or with the Z generator) gathered into
+// groups.  Such an
 // op may move anywhere between the ops that target its qubit (it commutes with
 // controls and other diagonals, and the gradient term of a generator Z does
 // not change across an op that commutes with it); groups are placed where the
@@ -225,7 +226,9 @@ int group_diagonals(const BOp* ops, int n, BOp* out) {
   };
   for (int i = 0; i < n; i++) {
     const BOp& z = ops[i];
-    if (z.kind != OPK_DIAG || z.k != 1 || z.lmask || z.xmask || (z.grad && !(z.flags & OPF_GZ))) continue;
+    if (z.kind != OPK_DIAG || z.k != 1 || z.lmask || z.xmask || !(z.flags & OPF_UNIT) ||
+        (z.grad && !(z.flags & OPF_GZ)))
+      continue;
     Range r{i, 0, n};
     for (int j = i - 1; j >= 0 && !r.first; j--)
       if (targets(j, z.gq[0])) r.first = j + 1;
@@ -363,6 +366,7 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
       if (op.k == 1 && op.kind == OPK_DENSE && G == Coefs{0.0, -j, j, 0.0}) d.flags |= OPF_REALM | OPF_GY;
       if (op.k == 1 && op.kind == OPK_DENSE && G == Coefs{0.0, 1.0, 1.0, 0.0}) d.flags |= OPF_GX;
       if (op.k == 1 && op.kind == OPK_DIAG && G == Coefs{1.0, -1.0}) d.flags |= OPF_GZ;
+      if (op.kind == OPK_DIAG) d.flags |= OPF_UNIT;
       d.table = 1;
       d.coef = (uint32_t)g.pidx;
       if (reverse) {
@@ -376,6 +380,11 @@ void fill_program(const std::vector<AGate>& ag, const std::vector<int>& order, c
       bool real = op.kind == OPK_DENSE;
       for (const cplx& v : op.m) real = real && v.imag() == 0.0;
       if (real) d.flags |= OPF_REALM;
+      // a matrix of the caller's may be off by 1e-6, which a group's table
+      // (brought back to modulus one) would drop
+      if (op.kind == OPK_DIAG && std::all_of(op.m.begin(), op.m.end(),
+                                             [](const cplx& v) { return std::abs(std::norm(v) - 1.0) < 1e-14; }))
+        d.flags |= OPF_UNIT;
       d.coef = (uint32_t)put(op.m);
     }
     P.ops[oi] = d;

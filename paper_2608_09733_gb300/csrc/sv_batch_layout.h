@@ -15,6 +15,7 @@ constexpr uint16_t OPF_REALM = 8;
 constexpr uint16_t OPF_GX = 16;
 constexpr uint16_t OPF_GY = 32;
 constexpr uint16_t OPF_GZ = 64;
+constexpr uint16_t OPF_UNIT = 128;  // a diagonal whose entries have modulus one to double rounding
 
 // ----------------------------------------------------------------- batched programs
 //
@@ -49,8 +50,8 @@ struct BOp {
 };
 static_assert(sizeof(BOp) == 64, "BOp layout");
 
-// A group of uncontrolled one-qubit diagonals of a register phase (RZ of any
-// qubits, S, T ...): a header of this kind with k = the members, which follow
+// A group of uncontrolled one-qubit diagonals of modulus one (OPF_UNIT) of a
+// register phase (RZ of any qubits, S, T ...): a header of this kind with k = the members, which follow
 // it as ops of their own.  Members on register slots make one table of 2^kRegQ
 // factors per state (at the header's soff), the others one factor a thread, so
 // psi and lambda are multiplied once for the whole group, and the gradient

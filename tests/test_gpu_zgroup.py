@@ -64,3 +64,21 @@ def test_gradients(svlib, cuda_dev, n, layers, ckpt, dtype):
     for b in range(3):
         v_ref, g_ref = oracle.adjoint_grad(n, gates, th[b], terms, npar)
         assert abs(v[b] - v_ref) < TOL[dtype] and np.abs(g[b] - g_ref).max() < TOL[dtype]
+
+
+@pytest.mark.parametrize("qubits", [[11], [0, 5, 11]])
+def test_a_callers_matrix_keeps_its_modulus(svlib, cuda_dev, qubits):
+    # accepted within 1e-6 of unitary: modulus 1 + 4e-7 forty times over is
+    # 3.2e-5 in a value of order one, three times the single precision bound
+    # of its 120 operations (120 x 2^-24, of a norm squared)
+    n, tol = 12, 1e-5
+    big = np.diag([1.0 + 4e-7, (1.0 + 4e-7) * 1j])
+    gates = [Gate("ry", [q], slots=[q], params=[0.0]) for q in range(n)]
+    for k in range(40):
+        q = qubits[k % len(qubits)]
+        gates += [Gate("rz", [(q + 1) % n], slots=[n], params=[0.0]), Gate("unitary", [q], matrix=big)]
+    terms = [Term("ZZ", [1, 2], 1.0)]
+    th = np.full((2, n + 1), 0.3)
+    v, _ = sv.sv_adjoint_grad(n, sv.SV_C64, gates, th, terms)
+    v_ref, _ = oracle.adjoint_grad(n, gates, th[0], terms, n + 1)
+    assert np.abs(v - v_ref).max() < tol
