@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <complex>
 #include <memory>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -64,167 +65,28 @@ bool rot_split(const cplx* U, double tol, RotSplit& r) {
   return true;
 }
 
-// Converts one sweep of the plan into the kernel's program: each op gets local
-// positions and control masks; consecutive ops whose moving qubits fit four
-// register slots form one register phase; dense k >= 3 blocks and wide
-// diagonals get a shared-memory phase of their own.
-// order: 0 keeps the pass's op order, 1 orders by phases where the rule below
-// says so, 2 always.  False when the pass does not fit one program: the
-// scheduler counts its ops and their coefficients, not the tables, merged
-// groups and phases that are made of them here.
+// An op on its way into a program.
+struct Tmp {
+  DevOp d;
+  Coefs m;
+  bool smem;
+  uint32_t need;  // local positions that must be register slots
+};
+
+// The program of the ops `ts` in that order (attach: see build_program): register
+// phases, then the ops as the kernel runs them.  False when they do not fit one
+// program: the scheduler counts a pass's ops and their coefficients, not the
+// tables, merged groups and phases that are made of them here.
 template <typename R>
-bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override, int order_by) {
+bool finish_program(const Plan& plan, const Sweep& sw, int rq, std::vector<Tmp>& ts, const std::vector<int>& ts_attach,
+                    SweepProgram<R>& P) {
   std::memset(&P.h, 0, sizeof(P.h));
   P.h.n = plan.n;
   P.h.m = sw.m;
   P.h.L = sw.L;
-  const int rq = rq_override > 0 ? rq_override : plan.lane ? kMaxRegQ : reg_qubits_for(sw.m);
   P.h.rq = rq;
   P.h.lane = plan.lane ? 1 : 0;
-  P.h.nops = (int)sw.ops.size();
-  int loc[64];
-  for (int q = 0; q < 64; q++) loc[q] = -1;
-  for (int i = 0; i < sw.m; i++) {
-    P.h.tq[i] = (int8_t)sw.tq[i];
-    loc[sw.tq[i]] = i;
-  }
-  const bool reg_ok = sw.m >= rq && (plan.lane || sw.m - rq <= 8);
-  struct Tmp {
-    DevOp d;
-    Coefs m;
-    bool smem;
-    uint32_t need;  // local positions that must be register slots
-  };
-  // Op order inside the pass.  Diagonal ops commute with each other and with
-  // every op whose targets (not controls) avoid their qubits.  A narrow
-  // diagonal D may sit anywhere between the last earlier op that targets one
-  // of its qubits (a "blocker") and the first later one: every op in between
-  // commutes with it, whichever side of D it was on.  It is placed just
-  // before its first later blocker, so it lands in the phase where its qubits
-  // are register slots and joins that phase's table (attach = +1); the
-  // rotation grouping below may hoist it further, in front of a whole group.
-  // Without a later blocker it goes just after the run of uncontrolled
-  // one-qubit gates that holds its last earlier blocker (attach = -1).
-  const int nsw = (int)sw.ops.size();
-  std::vector<int> order(nsw), attach(nsw, 0);
-  {
-    auto is_diag = [&](int i) {
-      const LOp& op = plan.ops[sw.ops[i]];
-      return op.kind == OPK_DIAG && op.k <= 2;
-    };
-    auto is_u1 = [&](int i) {
-      const LOp& op = plan.ops[sw.ops[i]];
-      return (op.kind == OPK_DENSE || op.kind == OPK_REAL) && op.k == 1 && op.nc == 0;
-    };
-    auto targets = [&](int i) {
-      const LOp& op = plan.ops[sw.ops[i]];
-      uint64_t t = 0;
-      for (int j = 0; j < op.k; j++) t |= 1ull << op.q[j];
-      return t;
-    };
-    // end of the run of uncontrolled one-qubit gates (diagonals skipped) holding each op
-    std::vector<int> run_end(nsw);
-    int next = -1;
-    for (int i = nsw - 1; i >= 0; i--) {
-      if (is_diag(i)) continue;
-      run_end[i] = (next >= 0 && is_u1(i) && is_u1(next)) ? run_end[next] : i;
-      next = i;
-    }
-    std::vector<std::tuple<int, int, int>> key(nsw);  // (anchor, before/at/after, original index)
-    for (int i = 0; i < nsw; i++) {
-      key[i] = std::make_tuple(i, 1, i);
-      if (!is_diag(i)) continue;
-      const uint64_t qs = plan.ops[sw.ops[i]].touch;
-      int after = -1, before = -1;
-      for (int j = i - 1; j >= 0 && before < 0; j--)
-        if (!is_diag(j) && (targets(j) & qs)) before = j;
-      for (int j = i + 1; j < nsw && after < 0; j++)
-        if (!is_diag(j) && (targets(j) & qs)) after = j;
-      if (after >= 0) {
-        key[i] = std::make_tuple(after, 0, i);
-        attach[i] = 1;
-      } else if (before >= 0) {
-        key[i] = std::make_tuple(run_end[before], 2, i);
-        attach[i] = -1;
-      }
-    }
-    for (int i = 0; i < nsw; i++) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key[a] < key[b]; });
-    if (std::getenv("SV_DEBUG_PLAN") && std::getenv("SV_DEBUG_PLAN")[0] == '3') {
-      std::fprintf(stderr, "[sv order]");
-      for (int i = 0; i < nsw; i++) {
-        const LOp& op = plan.ops[sw.ops[order[i]]];
-        std::fprintf(stderr, " %s%d%s%d", is_diag(order[i]) ? "D" : "U", op.q[0], op.k > 1 ? "." : "", op.k > 1 ? op.q[1] : (op.nc ? op.c[0] : -1));
-        std::fprintf(stderr, "@%d", order[i]);
-      }
-      std::fprintf(stderr, "\n");
-    }
-  }
-  std::vector<Tmp> ts(sw.ops.size());
-  std::vector<int> ts_attach(nsw);
-  for (size_t oi = 0; oi < sw.ops.size(); oi++) {
-    const LOp& op = plan.ops[sw.ops[order[oi]]];
-    ts_attach[oi] = attach[order[oi]];
-    Tmp& t = ts[oi];
-    DevOp& d = t.d;
-    std::memset(&d, 0, sizeof(d));
-    d.kind = op.kind;
-    d.k = (uint8_t)op.k;
-    t.m = op.m;
-    t.need = 0;
-    for (int i = 0; i < 5; i++) d.rs[i] = 0xFF;
-    int sp[5], ns = 0;
-    const bool diag = op.kind == OPK_DIAG;
-    for (int i = 0; i < op.k; i++) {
-      int l = loc[op.q[i]];
-      d.gq[i] = (uint8_t)op.q[i];
-      if (diag) {
-        d.pos[i] = l < 0 ? 0xFF : (uint8_t)l;
-      } else {
-        if (l < 0) fail(SV_ERR_INVALID, "internal: target outside the tile");
-        d.pos[i] = (uint8_t)l;
-        sp[ns++] = l;
-        t.need |= 1u << l;
-      }
-    }
-    for (int i = 1; i < ns; i++)
-      for (int j = i; j > 0 && sp[j - 1] > sp[j]; j--) std::swap(sp[j], sp[j - 1]);
-    for (int i = 0; i < ns; i++) d.spos[i] = (uint8_t)sp[i];
-    for (int i = 0; i < op.nc; i++) {
-      int l = loc[op.c[i]];
-      if (l >= 0) {
-        d.lmask |= 1u << l;
-        if (op.cs[i]) d.lval |= 1u << l;
-      } else {
-        d.xmask |= 1ull << op.c[i];
-        if (op.cs[i]) d.xval |= 1ull << op.c[i];
-      }
-    }
-    if (diag) {
-      // diag(1, .., 1, -1): a sign flip where every matrix bit is 1 (Z, CZ, CCZ)
-      const int dd = 1 << op.k;
-      bool sign = true;
-      for (int r = 0; r < dd; r++)
-        if (op.m[r] != (r == dd - 1 ? cplx(-1.0) : cplx(1.0))) sign = false;
-      if (sign) {
-        d.kind = OPK_SIGN;
-        t.m.clear();
-        for (int i = 0; i < op.k; i++) {
-          if (d.pos[i] != 0xFF) {
-            d.lmask |= 1u << d.pos[i];
-            d.lval |= 1u << d.pos[i];
-          } else {
-            d.xmask |= 1ull << op.q[i];
-            d.xval |= 1ull << op.q[i];
-          }
-        }
-      }
-    }
-    if (op.kind == OPK_ANTIDIAG && op.m.size() == 2 && op.m[0] == cplx(1.0) && op.m[1] == cplx(1.0)) d.pad = 1;
-    const bool wide = (op.kind == OPK_DENSE || op.kind == OPK_REAL) ? op.k >= 3 : (diag && d.kind == OPK_DIAG && op.k >= 3);
-    t.smem = !reg_ok || wide;
-  }
-
+  for (int i = 0; i < sw.m; i++) P.h.tq[i] = (int8_t)sw.tq[i];
   // phases
   int nph = 0;
   bool fits = true;
@@ -288,41 +150,6 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
       }
     }
   };
-  // The order of the ops over the phases.  A phase takes, in order, every op
-  // whose moving qubits still fit its register slots and that commutes with
-  // each op passed over before it, not only the run of ops up to the first
-  // that does not fit: of two ops, the later may go first when on every qubit
-  // they share both act diagonally (as a control or a diagonal).  That takes
-  // about 40 % fewer phases and up to 30 % more tables (20 layers of U3 and CZ
-  // on 24 qubits: 63 phases and 178 tables; 22 layers of U3 and CNOT ladder on
-  // 17: 78 phases and 199 tables against 131 and 219).  Complex64 states of 25
-  // qubits and more stream from HBM in compiled passes, where a table
-  // costs as much as a phase: they take this order only where it saves three
-  // phases of a pass (a 30-qubit pass of 7 phases 7.85 ms, of 4 phases and
-  // three more tables 5.92; one of 4 phases 4.35 ms, of 3 phases and two more
-  // tables 4.80).
-  if (plan.carry_flips && order_by) {
-    const int nt = (int)ts.size();
-    std::vector<PhaseOp> pops(nt);
-    for (int o = 0; o < nt; o++) {
-      const LOp& op = plan.ops[sw.ops[order[o]]];
-      pops[o] = phase_op(op, ts[o].need, ts[o].smem);
-    }
-    int phases = 0, runs = 0;
-    const std::vector<int> seq = order_by_phase(pops, rq, &phases, &runs);
-    const bool streams = sizeof(R) == 4 && plan.n >= 25;
-    if (order_by == 2 || runs - phases >= (streams ? 3 : 1)) {
-      std::vector<Tmp> ts2;
-      std::vector<int> at2;
-      ts2.reserve(nt);
-      for (int o : seq) {
-        ts2.push_back(std::move(ts[o]));
-        at2.push_back(ts_attach[o]);
-      }
-      ts = std::move(ts2);
-      ts_attach = std::move(at2);
-    }
-  }
   // Greedy register phases.  Diagonals attached forward wait for their op and
   // open its phase with it; the others join the phase in progress.
   int cur_first = -1, cur_n = 0, pend = 0;
@@ -819,12 +646,191 @@ bool build_program_ordered(const Plan& plan, const Sweep& sw, SweepProgram<R>& P
   return true;
 }
 
-// Complex128 passes of many tiles are bound by the FP64 pipe: a table is four
-// instructions an amplitude, a phase none, so both orders are built and the
-// one with fewer tables is kept (by less than two phases a table).
+// Converts one sweep of the plan into the kernel's program: each op gets local
+// positions and control masks; consecutive ops whose moving qubits fit four
+// register slots form one register phase; dense k >= 3 blocks and wide
+// diagonals get a shared-memory phase of their own.  False when the sweep does
+// not fit one program.
 template <typename R>
 bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override) {
-  if (!(sizeof(R) == 8 && plan.carry_flips && !plan.lane)) return build_program_ordered<R>(plan, sw, P, rq_override, 1);
+  const int rq = rq_override > 0 ? rq_override : plan.lane ? kMaxRegQ : reg_qubits_for(sw.m);
+  int loc[64];
+  for (int q = 0; q < 64; q++) loc[q] = -1;
+  for (int i = 0; i < sw.m; i++) loc[sw.tq[i]] = i;
+  const bool reg_ok = sw.m >= rq && (plan.lane || sw.m - rq <= 8);
+  // Op order inside the pass.  Diagonal ops commute with each other and with
+  // every op whose targets (not controls) avoid their qubits.  A narrow
+  // diagonal D may sit anywhere between the last earlier op that targets one
+  // of its qubits (a "blocker") and the first later one: every op in between
+  // commutes with it, whichever side of D it was on.  It is placed just
+  // before its first later blocker, so it lands in the phase where its qubits
+  // are register slots and joins that phase's table (attach = +1); the
+  // rotation grouping below may hoist it further, in front of a whole group.
+  // Without a later blocker it goes just after the run of uncontrolled
+  // one-qubit gates that holds its last earlier blocker (attach = -1).
+  const int nsw = (int)sw.ops.size();
+  std::vector<int> order(nsw), attach(nsw, 0);
+  {
+    auto is_diag = [&](int i) {
+      const LOp& op = plan.ops[sw.ops[i]];
+      return op.kind == OPK_DIAG && op.k <= 2;
+    };
+    auto is_u1 = [&](int i) {
+      const LOp& op = plan.ops[sw.ops[i]];
+      return (op.kind == OPK_DENSE || op.kind == OPK_REAL) && op.k == 1 && op.nc == 0;
+    };
+    auto targets = [&](int i) {
+      const LOp& op = plan.ops[sw.ops[i]];
+      uint64_t t = 0;
+      for (int j = 0; j < op.k; j++) t |= 1ull << op.q[j];
+      return t;
+    };
+    // end of the run of uncontrolled one-qubit gates (diagonals skipped) holding each op
+    std::vector<int> run_end(nsw);
+    int next = -1;
+    for (int i = nsw - 1; i >= 0; i--) {
+      if (is_diag(i)) continue;
+      run_end[i] = (next >= 0 && is_u1(i) && is_u1(next)) ? run_end[next] : i;
+      next = i;
+    }
+    std::vector<std::tuple<int, int, int>> key(nsw);  // (anchor, before/at/after, original index)
+    for (int i = 0; i < nsw; i++) {
+      key[i] = std::make_tuple(i, 1, i);
+      if (!is_diag(i)) continue;
+      const uint64_t qs = plan.ops[sw.ops[i]].touch;
+      int after = -1, before = -1;
+      for (int j = i - 1; j >= 0 && before < 0; j--)
+        if (!is_diag(j) && (targets(j) & qs)) before = j;
+      for (int j = i + 1; j < nsw && after < 0; j++)
+        if (!is_diag(j) && (targets(j) & qs)) after = j;
+      if (after >= 0) {
+        key[i] = std::make_tuple(after, 0, i);
+        attach[i] = 1;
+      } else if (before >= 0) {
+        key[i] = std::make_tuple(run_end[before], 2, i);
+        attach[i] = -1;
+      }
+    }
+    for (int i = 0; i < nsw; i++) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key[a] < key[b]; });
+    if (std::getenv("SV_DEBUG_PLAN") && std::getenv("SV_DEBUG_PLAN")[0] == '3') {
+      std::fprintf(stderr, "[sv order]");
+      for (int i = 0; i < nsw; i++) {
+        const LOp& op = plan.ops[sw.ops[order[i]]];
+        std::fprintf(stderr, " %s%d%s%d", is_diag(order[i]) ? "D" : "U", op.q[0], op.k > 1 ? "." : "", op.k > 1 ? op.q[1] : (op.nc ? op.c[0] : -1));
+        std::fprintf(stderr, "@%d", order[i]);
+      }
+      std::fprintf(stderr, "\n");
+    }
+  }
+  std::vector<Tmp> ts(sw.ops.size());
+  std::vector<int> ts_attach(nsw);
+  for (size_t oi = 0; oi < sw.ops.size(); oi++) {
+    const LOp& op = plan.ops[sw.ops[order[oi]]];
+    ts_attach[oi] = attach[order[oi]];
+    Tmp& t = ts[oi];
+    DevOp& d = t.d;
+    std::memset(&d, 0, sizeof(d));
+    d.kind = op.kind;
+    d.k = (uint8_t)op.k;
+    t.m = op.m;
+    t.need = 0;
+    for (int i = 0; i < 5; i++) d.rs[i] = 0xFF;
+    int sp[5], ns = 0;
+    const bool diag = op.kind == OPK_DIAG;
+    for (int i = 0; i < op.k; i++) {
+      int l = loc[op.q[i]];
+      d.gq[i] = (uint8_t)op.q[i];
+      if (diag) {
+        d.pos[i] = l < 0 ? 0xFF : (uint8_t)l;
+      } else {
+        if (l < 0) fail(SV_ERR_INVALID, "internal: target outside the tile");
+        d.pos[i] = (uint8_t)l;
+        sp[ns++] = l;
+        t.need |= 1u << l;
+      }
+    }
+    for (int i = 1; i < ns; i++)
+      for (int j = i; j > 0 && sp[j - 1] > sp[j]; j--) std::swap(sp[j], sp[j - 1]);
+    for (int i = 0; i < ns; i++) d.spos[i] = (uint8_t)sp[i];
+    for (int i = 0; i < op.nc; i++) {
+      int l = loc[op.c[i]];
+      if (l >= 0) {
+        d.lmask |= 1u << l;
+        if (op.cs[i]) d.lval |= 1u << l;
+      } else {
+        d.xmask |= 1ull << op.c[i];
+        if (op.cs[i]) d.xval |= 1ull << op.c[i];
+      }
+    }
+    if (diag) {
+      // diag(1, .., 1, -1): a sign flip where every matrix bit is 1 (Z, CZ, CCZ)
+      const int dd = 1 << op.k;
+      bool sign = true;
+      for (int r = 0; r < dd; r++)
+        if (op.m[r] != (r == dd - 1 ? cplx(-1.0) : cplx(1.0))) sign = false;
+      if (sign) {
+        d.kind = OPK_SIGN;
+        t.m.clear();
+        for (int i = 0; i < op.k; i++) {
+          if (d.pos[i] != 0xFF) {
+            d.lmask |= 1u << d.pos[i];
+            d.lval |= 1u << d.pos[i];
+          } else {
+            d.xmask |= 1ull << op.q[i];
+            d.xval |= 1ull << op.q[i];
+          }
+        }
+      }
+    }
+    if (op.kind == OPK_ANTIDIAG && op.m.size() == 2 && op.m[0] == cplx(1.0) && op.m[1] == cplx(1.0)) d.pad = 1;
+    const bool wide = (op.kind == OPK_DENSE || op.kind == OPK_REAL) ? op.k >= 3 : (diag && d.kind == OPK_DIAG && op.k >= 3);
+    t.smem = !reg_ok || wide;
+  }
+
+  // The order of the ops over the phases.  A phase takes, in order, every op
+  // whose moving qubits still fit its register slots and that commutes with
+  // each op passed over before it, not only the run of ops up to the first
+  // that does not fit: of two ops, the later may go first when on every qubit
+  // they share both act diagonally (as a control or a diagonal).  That takes
+  // about 40 % fewer phases and up to 30 % more tables (20 layers of U3 and CZ
+  // on 24 qubits: 63 phases and 178 tables; 22 layers of U3 and CNOT ladder on
+  // 17: 78 phases and 199 tables against 131 and 219).  Complex64 states of 25
+  // qubits and more stream from HBM in compiled passes, where a table
+  // costs as much as a phase: they take this order only where it saves three
+  // phases of a pass (20 layers of U3 and CZ on 28 qubits, 33 passes: in order
+  // 112 phases and 158 tables 29.0 ms, so 109 and 162 28.8, always 76 and 204
+  // 29.8).
+  // Complex128 passes of many tiles are bound by the FP64 pipe: a table is four
+  // instructions an amplitude, a phase none.  Without bit flips or swaps to
+  // carry tables across, this order has more tables and they keep the given one
+  // (20 layers of U3 and CZ on 20 qubits: 127 tables 3.24 ms, 159 3.56).
+  const bool fp64 = sizeof(R) == 8 && !plan.lane;
+  const int nt = (int)ts.size();
+  bool flips = false;
+  std::vector<PhaseOp> pops(nt);
+  for (int o = 0; o < nt; o++) {
+    const LOp& op = plan.ops[sw.ops[order[o]]];
+    pops[o] = phase_op(op, ts[o].need, ts[o].smem);
+    flips = flips || op.kind == OPK_ANTIDIAG || op.kind == OPK_SWAP;
+  }
+  if (!plan.carry_flips || (fp64 && !flips)) return finish_program<R>(plan, sw, rq, ts, ts_attach, P);
+  int phases = 0, runs = 0;
+  const std::vector<int> seq = order_by_phase(pops, rq, &phases, &runs);
+  std::vector<int> attach2;
+  attach2.reserve(nt);
+  for (int o : seq) attach2.push_back(ts_attach[o]);
+  std::vector<Tmp> ts2;
+  ts2.reserve(nt);
+  if (!fp64) {
+    const bool streams = sizeof(R) == 4 && plan.n >= 25;
+    if (runs - phases < (streams ? 3 : 1)) return finish_program<R>(plan, sw, rq, ts, ts_attach, P);
+    for (int o : seq) ts2.push_back(std::move(ts[o]));
+    return finish_program<R>(plan, sw, rq, ts2, attach2, P);
+  }
+  // With flips both orders are made, and the one with fewer tables is kept (by
+  // less than two phases a table): 10 layers of U3 and CNOT ladder on 20
+  // qubits, 152 tables in order 2.57 ms, 127 by phases 2.33.
   auto cost = [](const SweepProgram<R>& p) {
     int tables = 0;
     for (int i = 0; i < p.h.nphases; i++)
@@ -832,10 +838,12 @@ bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
         for (int o = p.ph[i].first; o < p.ph[i].first + p.ph[i].nops; o++) tables += (p.ops[o].pad & 15u) == OPK_PHASE;
     return 2 * tables + p.h.nphases;
   };
-  std::unique_ptr<SweepProgram<R>> other(new SweepProgram<R>());
-  const bool fits = build_program_ordered<R>(plan, sw, P, rq_override, 0);
-  const bool other_fits = build_program_ordered<R>(plan, sw, *other, rq_override, 2);
-  if (other_fits && (!fits || cost(*other) < cost(P))) std::memcpy(&P, other.get(), sizeof(P));
+  for (int o : seq) ts2.push_back(ts[o]);
+  std::unique_ptr<SweepProgram<R>> other(new SweepProgram<R>);
+  const bool fits = finish_program<R>(plan, sw, rq, ts, ts_attach, P);
+  const bool other_fits = finish_program<R>(plan, sw, rq, ts2, attach2, *other);
+  if (other_fits && (!fits || cost(*other) < cost(P)))
+    std::memcpy(&P, other.get(), offsetof(SweepProgram<R>, coef) + sizeof(Cx<R>) * other->h.ncoef);
   return fits || other_fits;
 }
 
