@@ -420,7 +420,7 @@ PhaseOp phase_op(const LOp& op, uint32_t need, bool smem) {
 // With `commute` an op may go before ops passed over when on every qubit it
 // shares with them both act diagonally (controls and diagonals commute), not
 // only when it shares none: CZ layers then hold up fewer ops (20 layers of U3
-// and CZ on 30 qubits: 35 passes against 38, on 24 qubits 25 against 28).
+// and CZ on 30 qubits: 35 passes against 38, on 24 qubits 26 against 28).
 std::vector<Sweep> schedule_sweeps(int n, const std::vector<const LOp*>& ops, int tile_q, int low_q, int coef_pool,
                                    int ops_per_pass, bool commute) {
   const int max_ops = ops_per_pass > 0 ? std::min(ops_per_pass, kMaxOps) : kMaxOps;
@@ -786,26 +786,48 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
   // has more tables (20 layers of U3 and CZ on 24 qubits: 28 passes 48.3 ms,
   // 29 passes 46.3).
   const bool commute = tile_q_override == 0 && (dtype == SV_C64 || lane);
-  auto schedule = [&](const std::vector<LOp>& ops) {
+  auto schedule = [&](const std::vector<LOp>& ops, bool by_commuting) {
     std::vector<const LOp*> list;
     list.reserve(ops.size());
     for (const LOp& op : ops) list.push_back(&op);
-    return schedule_sweeps(n, list, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass, commute);
+    return schedule_sweeps(n, list, tile_q, low_qubits_for(dtype), pool, opts.ops_per_pass, by_commuting);
   };
-  p.sweeps = schedule(p.ops);
+  p.sweeps = schedule(p.ops, commute);
   if (opts.ops_per_pass != 1) {
     // The split form has more ops, which can cut the greedy passes short and
-    // leave more of them: keep it only when it needs no more passes, or at most
-    // one in twenty more.  Whole gates close with a table of their own in each
-    // phase: 20 layers of U3 and CZ on 28 qubits take 31.8 ms with 32 passes
-    // and 252 tables, 28.7 ms with 33 passes and 162.
+    // leave more of them: keep it only when it needs no more passes, or a few
+    // more for the tables it saves.  Whole gates close with a table of their
+    // own in each phase, so what it saves goes with the gates that split: one
+    // pass more for a hundred of them, up to one in twenty, or one in five
+    // where the passes run compiled (a table is a larger part of those).
+    // Complex64, U3 and CZ, whole against split: 28 qubits, 20 layers, 32
+    // passes and 252 tables 31.7 ms, 33 and 162 28.8; 26 qubits, 8 layers, 10
+    // and 90 3.18 ms, 11 and 69 3.04; interpreted, 18 qubits, 20 layers, 8 and
+    // 148 233 us, 12 and 136 259.  A CNOT ladder splits the gates of one qubit
+    // only (21 qubits, 10 layers: 21 passes and 120 tables 339 us, 22 and 119
+    // 348).
+    const bool compiled = commute && !lane && n >= SV_C64_TMA_MIN_N;
     std::vector<LOp> ops2 = split_one_qubit(p.ops, dtype == SV_C64 ? 1e-9 : 1e-13);
+    const size_t nsplit = ops2.size() - p.ops.size();
     drop_identities(ops2);
-    std::vector<Sweep> sw2 = schedule(ops2);
-    const size_t more = commute ? p.sweeps.size() / 20 : 0;
+    std::vector<Sweep> sw2 = schedule(ops2, commute);
+    const size_t more = commute ? std::min(nsplit / 100, p.sweeps.size() / (compiled ? 5 : 20)) : 0;
     if (sw2.size() <= p.sweeps.size() + more) {
       p.ops = std::move(ops2);
       p.sweeps = std::move(sw2);
+    }
+    // States that stream from HBM take the passes in the given order where
+    // ordering by what commutes saves a single pass of twelve or more: the
+    // fewer passes hold more tables, and a table costs there what a fifth of a
+    // pass does.  Complex64, U3 and CZ, in order against commuting: 26 qubits,
+    // 8 layers, 12 passes and 63 tables 2.90 ms, 11 and 69 3.04; 25 qubits, 18
+    // layers, 26 and 119 3.24 ms, 25 and 133 3.30; but 26 qubits, 16 layers, 25
+    // and 113 5.83 ms, 23 and 124 5.74; 28 qubits, 20 layers, 35 and 152 29.8
+    // ms, 33 and 162 28.8; 27 qubits, 5 layers, 9 and 45 3.96 ms, 8 and 46 3.86.
+    if (compiled && n >= 25) {
+      std::vector<Sweep> in_order = schedule(p.ops, false);
+      const size_t saved = in_order.size() - std::min(in_order.size(), p.sweeps.size());
+      if (saved < 2 && saved * 11 < in_order.size()) p.sweeps = std::move(in_order);
     }
     defer_diagonals(p.ops, p.sweeps, max_ops, pool);
   }
