@@ -804,7 +804,9 @@ bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
   // Complex128 passes of many tiles are bound by the FP64 pipe: a table is four
   // instructions an amplitude, a phase none.  Without bit flips or swaps to
   // carry tables across, this order has more tables and they keep the given one
-  // (20 layers of U3 and CZ on 20 qubits: 127 tables 3.24 ms, 159 3.56).
+  // (20 layers of U3 and CZ on 20 qubits: 127 tables 3.20 ms, 159 3.56), but
+  // for passes it leaves two phases, which have as many tables either way (7 of
+  // the 25: 3.18 ms).
   const bool fp64 = sizeof(R) == 8 && !plan.lane;
   const int nt = (int)ts.size();
   bool flips = false;
@@ -814,7 +816,7 @@ bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
     pops[o] = phase_op(op, ts[o].need, ts[o].smem);
     flips = flips || op.kind == OPK_ANTIDIAG || op.kind == OPK_SWAP;
   }
-  if (!plan.carry_flips || (fp64 && !flips)) return finish_program<R>(plan, sw, rq, ts, ts_attach, P);
+  if (!plan.carry_flips) return finish_program<R>(plan, sw, rq, ts, ts_attach, P);
   int phases = 0, runs = 0;
   const std::vector<int> seq = order_by_phase(pops, rq, &phases, &runs);
   std::vector<int> attach2;
@@ -822,9 +824,10 @@ bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq
   for (int o : seq) attach2.push_back(ts_attach[o]);
   std::vector<Tmp> ts2;
   ts2.reserve(nt);
-  if (!fp64) {
+  if (!fp64 || !flips) {
     const bool streams = sizeof(R) == 4 && plan.n >= 25;
-    if (runs - phases < (streams ? 3 : 1)) return finish_program<R>(plan, sw, rq, ts, ts_attach, P);
+    const bool keep = fp64 ? phases > 2 || runs - phases < 2 : runs - phases < (streams ? 3 : 1);
+    if (keep) return finish_program<R>(plan, sw, rq, ts, ts_attach, P);
     for (int o : seq) ts2.push_back(std::move(ts[o]));
     return finish_program<R>(plan, sw, rq, ts2, attach2, P);
   }
