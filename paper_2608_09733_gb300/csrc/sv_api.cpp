@@ -21,6 +21,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <shared_mutex>
 #include <thread>
 #include <tuple>
 
@@ -225,6 +226,7 @@ namespace {
 struct Compiled {
   std::vector<unsigned char> key;
   int n = 0;
+  bool lane = false;  // programs of the cluster pass
   std::vector<SweepProgram<float>> pf;
   std::vector<SweepProgram<double>> pd;
   // the programs' structure keys (sv_jit.cpp), made on the first run
@@ -264,8 +266,7 @@ std::vector<unsigned char> circuit_key(int n, sv_dtype dtype, const sv_gate* gat
 }
 
 std::shared_ptr<const Compiled> compiled_circuit(int n, sv_dtype dtype, const sv_gate* gates, size_t ng,
-                                                 const double* pv, size_t npv, const sv_exec_opts& opts) {
-  const bool lane = lane_sizes(n, opts) && lane_pass_available();
+                                                 const double* pv, size_t npv, const sv_exec_opts& opts, bool lane) {
   std::vector<unsigned char> key = circuit_key(n, dtype, gates, ng, pv, npv, opts, lane);
   {
     std::lock_guard<std::mutex> lk(g_compiled_mu);
@@ -280,6 +281,7 @@ std::shared_ptr<const Compiled> compiled_circuit(int n, sv_dtype dtype, const sv
   Plan plan = make_plan(n, dtype, gates, ng, pv, npv, opts, 0, lane);
   auto c = std::make_shared<Compiled>();
   c->n = n;
+  c->lane = lane;
   if (dtype == SV_C64)
     build_programs<float>(plan, c->pf);
   else
@@ -333,6 +335,34 @@ void run_compiled(void* state, const Compiled& c, sv_dtype dtype, cudaStream_t s
   }
 }
 
+// A circuit planned for the pass its state takes now, and run.  A cluster pass
+// is not enqueued beside a live serving session, whose resident CTAs could keep
+// its clusters of 16 waiting: sessions start under the gate held here, and one
+// that started since the plan was made has the circuit planned for the general
+// pass instead.  (A cluster pass already enqueued when a session starts may
+// still wait for it.)
+struct PlannedCircuit {
+  int n;
+  sv_dtype dtype;
+  const sv_gate* gates;
+  size_t ng;
+  const double* pv;
+  size_t npv;
+  const sv_exec_opts& opts;
+  std::shared_ptr<const Compiled> c;
+
+  void plan(bool lane) { c = compiled_circuit(n, dtype, gates, ng, pv, npv, opts, lane); }
+  void plan() { plan(lane_sizes(n, opts) && lane_pass_available()); }
+  void run(void* state, cudaStream_t stream) {
+    if (c->lane) {
+      std::shared_lock<std::shared_mutex> gate(session_gate());
+      if (lane_pass_available()) return run_compiled(state, *c, dtype, stream);
+    }
+    if (c->lane) plan(false);
+    run_compiled(state, *c, dtype, stream);
+  }
+};
+
 sv_exec_opts opts_of(const sv_exec_opts* o) {
   sv_exec_opts r;
   std::memset(&r, 0, sizeof(r));
@@ -348,7 +378,9 @@ sv_exec_opts fuse_opts(int fuse) {
 
 void apply_circuit(void* state, int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, const double* pv,
                    size_t npv, const sv_exec_opts& opts, cudaStream_t stream) {
-  run_compiled(state, *compiled_circuit(n, dtype, gates, n_gates, pv, npv, opts), dtype, stream);
+  PlannedCircuit p{n, dtype, gates, n_gates, pv, npv, opts, nullptr};
+  p.plan();
+  p.run(state, stream);
 }
 
 void expect_z_all_dev(const void* state, int n, sv_dtype dtype, double* out_dev, cudaStream_t stream) {
@@ -504,8 +536,9 @@ sv_status sv_run_host(int n_qubits, sv_dtype dtype, const void* state_in, const 
   return guarded([&] {
     check_dtype_n(n_qubits, dtype);
     if (!out_z) fail(SV_ERR_INVALID, "out_z is NULL");
-    std::shared_ptr<const Compiled> prog =
-        compiled_circuit(n_qubits, dtype, gates, n_gates, param_values, n_param_values, fuse_opts(fuse_max_k));
+    const sv_exec_opts opts = fuse_opts(fuse_max_k);
+    PlannedCircuit prog{n_qubits, dtype, gates, n_gates, param_values, n_param_values, opts, nullptr};
+    prog.plan();
     cudaStream_t s = (cudaStream_t)stream;
     const size_t bytes = amp_bytes(dtype) << n_qubits;
     Workspace& w = workspace(s, expect_z_all_scratch_doubles(n_qubits), n_qubits + 1, bytes);
@@ -516,7 +549,7 @@ sv_status sv_run_host(int n_qubits, sv_dtype dtype, const void* state_in, const 
     } else {
       cuda_check(launch_init_basis<double>((Cx<double>*)w.state, n_qubits, 0, s), "init launch");
     }
-    run_compiled(w.state, *prog, dtype, s);
+    prog.run(w.state, s);
     expect_z_all_dev(w.state, n_qubits, dtype, w.out, s);
     cuda_check(cudaMemcpyAsync(out_z, w.out, (n_qubits + 1) * sizeof(double), cudaMemcpyDeviceToHost, s),
                "result copy");

@@ -9,6 +9,7 @@
 #include <complex>
 #include <initializer_list>
 #include <memory>
+#include <shared_mutex>
 #include <string>
 #include <vector>
 
@@ -269,6 +270,8 @@ cudaError_t launch_small_session(const SmallSessionDev& d, const SweepProgram<R>
 void session_opened(int device, int ctas);
 void session_closed(int device, int ctas);
 bool session_live(int device);
+// Held shared while a cluster pass is enqueued, exclusively while a session starts.
+std::shared_mutex& session_gate();
 // Ends the kernels of the device's live sessions and holds them (their locks)
 // until sessions_release, which relaunches those with requests not done
 // (sv_serve.cpp): a module load waits for every resident kernel to end.

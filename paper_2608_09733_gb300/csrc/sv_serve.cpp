@@ -320,8 +320,16 @@ extern "C" sv_status sv_small_session_start(sv_dtype dtype, int capacity, int ar
     s->status = (int*)((char*)s->head + 16);
     cuda_check(cudaMemsetAsync(s->head, 0, 64, s->copy), "cudaMemset");
     cuda_check(cudaStreamSynchronize(s->copy), "cudaStreamSynchronize");
-    launch(s.get());
-    session_opened(s->device, s->grid);
+    {
+      std::unique_lock<std::shared_mutex> gate(session_gate());
+      session_opened(s->device, s->grid);
+      try {
+        launch(s.get());
+      } catch (...) {
+        session_closed(s->device, s->grid);
+        throw;
+      }
+    }
     {
       std::lock_guard<std::mutex> lk(g_sessions_mu);
       g_sessions.push_back(s.get());

@@ -798,6 +798,10 @@ void session_closed(int device, int ctas) {
   g_live_sessions[device]--;
   g_session_ctas[device] -= ctas;
 }
+std::shared_mutex& session_gate() {
+  static std::shared_mutex m;
+  return m;
+}
 bool session_live(int device) { return device >= 0 && device < 64 && g_live_sessions[device].load() > 0; }
 
 static bool tma_enabled() {
