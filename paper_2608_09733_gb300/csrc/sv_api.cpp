@@ -510,18 +510,7 @@ sv_status sv_plan_info(int n_qubits, sv_dtype dtype, const sv_gate* gates, size_
   return guarded([&] {
     const sv_exec_opts o = opts_of(opts);
     Plan plan = make_plan(n_qubits, dtype, gates, n_gates, param_values, n_param_values, o, 0, lane_sizes(n_qubits, o));
-    // the passes that run: a pass of the plan can take more than one program
-    // (SV_DEBUG_PLAN prints each)
-    size_t passes = 0;
-    if (dtype == SV_C64) {
-      std::vector<SweepProgram<float>> progs;
-      build_programs<float>(plan, progs);
-      passes = progs.size();
-    } else {
-      std::vector<SweepProgram<double>> progs;
-      build_programs<double>(plan, progs);
-      passes = progs.size();
-    }
+    const size_t passes = dtype == SV_C64 ? count_programs<float>(plan) : count_programs<double>(plan);
     int nb = (int)plan.block_starts.size() - 1;
     if (out_blocks) *out_blocks = nb;
     if (out_sweeps) *out_sweeps = (int)passes;

@@ -212,6 +212,10 @@ std::vector<int> order_by_phase(const std::vector<PhaseOp>& ops, int rq, int* ph
 // where a pass does not fit one.
 template <typename R>
 void build_programs(const Plan& plan, std::vector<SweepProgram<R>>& out, int rq_override = 0);
+// How many build_programs makes (the passes that run), building only those that
+// could be more than one.
+template <typename R>
+size_t count_programs(const Plan& plan);
 
 // ----------------------------------------------------------------- launches
 // (sv_sweep.cu / sv_reduce.cu).  All return cudaError_t of the launch.

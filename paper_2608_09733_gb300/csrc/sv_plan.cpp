@@ -722,13 +722,18 @@ static void defer_diagonals(const std::vector<LOp>& ops, std::vector<Sweep>& sw,
 
 // States of up to four cluster tiles (2^14 amplitudes each) take the cluster
 // pass: a tile spread over a cluster's SMs, an amplitude a lane.  At 17 qubits
-// the eight clusters no longer fit beside each other and the one-CTA tiles,
-// 16 of them by then, are faster (measured before phases were ordered;
-// complex64, U3 + CNOT ladder of depth 22: 15 qubits 430 against 461 us, 16
-// qubits 472 against 465 but 287 against 456 on random two-qubit matrices, 17
-// qubits 840 against 552).  Below five
-// qubits there is no warp to fill.  An explicit tile width or cap of
-// operations per pass keeps its own kernel.
+// the eight clusters no longer fit beside each other.  Cluster against general
+// pass, us a circuit, both with ordered phases:
+//                               16 qubits               17 qubits
+//                         complex64   complex128  complex64   complex128
+//   U3, CNOT ladder, 22   350   414    811  1485  569   495  1476  1494
+//   U3 and CZ, 20 layers  208   200    601   827  295   214  1196   910
+//   random, 300 matrices  125   254    463   945  194   259   872   981
+//   RY RZ CNOT, 10 layers 198   260    444   617  265   281   729   688
+// (14 and 15 qubits as 16: the cluster pass ahead but for U3 and CZ on 15
+// qubits in complex64, 201 against 191.)  Below five qubits there is no warp to
+// fill.  An explicit tile width or cap of operations per pass keeps its own
+// kernel.
 bool lane_sizes(int n, const sv_exec_opts& opts) {
   return n >= 5 && n <= 16 && opts.tile_qubits == 0 && opts.ops_per_pass == 0;
 }

@@ -872,6 +872,40 @@ void build_programs(const Plan& plan, std::vector<SweepProgram<R>>& out, int rq_
   for (const Sweep& sw : plan.sweeps) build_parts<R>(plan, sw, out, rq_override);
 }
 
+// Whether a pass fits one program whatever is made of it: the plain form at the
+// end of finish_program's tries has no more ops than the pass, and of its
+// coefficients only merged runs of one-qubit gates (two of them at least) take
+// more than the ops' own.
+template <typename R>
+static bool surely_fits(const Plan& plan, const Sweep& sw) {
+  int coef = 0, one = 0;
+  for (int i : sw.ops) {
+    const LOp& op = plan.ops[i];
+    coef += (int)op.m.size();
+    one += (op.kind == OPK_DENSE || op.kind == OPK_REAL) && op.k == 1;
+  }
+  return coef + one / 2 * (4 * kMaxRegQ - 8) <= SweepProgram<R>::kPool && (int)sw.ops.size() <= kMaxOps;
+}
+
+template <typename R>
+size_t count_programs(const Plan& plan) {
+  static const bool debug = std::getenv("SV_DEBUG_PLAN") != nullptr;  // prints the programs it builds
+  size_t n = 0;
+  std::vector<SweepProgram<R>> parts;
+  for (const Sweep& sw : plan.sweeps) {
+    if (!debug && surely_fits<R>(plan, sw)) {
+      n++;
+      continue;
+    }
+    parts.clear();
+    build_parts<R>(plan, sw, parts, 0);
+    n += parts.size();
+  }
+  return n;
+}
+
+template size_t count_programs<float>(const Plan&);
+template size_t count_programs<double>(const Plan&);
 template void build_programs<float>(const Plan&, std::vector<SweepProgram<float>>&, int);
 template void build_programs<double>(const Plan&, std::vector<SweepProgram<double>>&, int);
 
