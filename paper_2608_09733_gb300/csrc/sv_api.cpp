@@ -281,7 +281,7 @@ std::shared_ptr<const Compiled> compiled_circuit(int n, sv_dtype dtype, const sv
   Plan plan = make_plan(n, dtype, gates, ng, pv, npv, opts, 0, lane);
   auto c = std::make_shared<Compiled>();
   c->n = n;
-  c->lane = lane;
+  c->lane = plan.lane;
   if (dtype == SV_C64)
     build_programs<float>(plan, c->pf);
   else

@@ -731,11 +731,25 @@ static void defer_diagonals(const std::vector<LOp>& ops, std::vector<Sweep>& sw,
 //   random, 300 matrices  125   254    463   945  194   259   872   981
 //   RY RZ CNOT, 10 layers 198   260    444   617  265   281   729   688
 // (14 and 15 qubits as 16: the cluster pass ahead but for U3 and CZ on 15
-// qubits in complex64, 201 against 191.)  Below five qubits there is no warp to
+// qubits in complex64, 201 against 191; make_plan leaves short circuits of that
+// kind to the general pass.)  Below five qubits there is no warp to
 // fill.  An explicit tile width or cap of operations per pass keeps its own
 // kernel.
 bool lane_sizes(int n, const sv_exec_opts& opts) {
   return n >= 5 && n <= 16 && opts.tile_qubits == 0 && opts.ops_per_pass == 0;
+}
+
+// Complex64 states of two and four cluster tiles (15 and 16 qubits): a short
+// circuit of one-qubit gates and diagonals takes the general pass, whose one or
+// two wider passes run few phases.  U3 and CZ on 16 qubits, us, cluster against
+// general: 2 layers (62 gates) 36.9 and 28.6, 5 layers (155) 66.5 and 51.7, 6
+// layers (186) 65.9 and 64.1, then within a tenth (20 layers 208 and 200); with
+// flips (RY RZ CNOT, 1 layer) 28.0 and 31.6, with two-qubit matrices 20.8 and
+// 35.3.  The line is at 200 operations.
+static bool short_without_flips(const std::vector<LOp>& ops) {
+  return ops.size() < 200 && std::all_of(ops.begin(), ops.end(), [](const LOp& op) {
+           return op.kind == OPK_DIAG || ((op.kind == OPK_DENSE || op.kind == OPK_REAL) && op.k == 1);
+         });
 }
 
 Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, const double* param_values,
@@ -753,7 +767,6 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
   validate_gates(n, gates, n_gates, n_param_values);
   Plan p;
   p.n = n;
-  p.lane = lane;
   p.carry_flips = tile_q_override == 0;
   if (fuse_max_k >= 2) {
     p.ops = fuse_greedy(n, gates, n_gates, param_values, fuse_max_k, &p.block_starts,
@@ -780,6 +793,7 @@ Plan make_plan(int n, sv_dtype dtype, const sv_gate* gates, size_t n_gates, cons
     join_one_qubit(p.ops);
     drop_identities(p.ops);
   }
+  lane = p.lane = lane && !(dtype == SV_C64 && n > kMaxTileQ && short_without_flips(p.ops));
   int pool = dtype == SV_C64 ? SweepProgram<float>::kPool : SweepProgram<double>::kPool;
   const int tile_q = tile_q_override > 0 ? tile_q_override
                      : lane              ? std::min(n, kMaxTileQ)
