@@ -65,6 +65,7 @@ bool rot_split(const cplx* U, double tol, RotSplit& r) {
   return true;
 }
 
+namespace {
 // An op on its way into a program.
 struct Tmp {
   DevOp d;
@@ -72,14 +73,15 @@ struct Tmp {
   bool smem;
   uint32_t need;  // local positions that must be register slots
 };
+}  // namespace
 
 // The program of the ops `ts` in that order (attach: see build_program): register
 // phases, then the ops as the kernel runs them.  False when they do not fit one
 // program: the scheduler counts a pass's ops and their coefficients, not the
 // tables, merged groups and phases that are made of them here.
 template <typename R>
-bool finish_program(const Plan& plan, const Sweep& sw, int rq, std::vector<Tmp>& ts, const std::vector<int>& ts_attach,
-                    SweepProgram<R>& P) {
+static bool finish_program(const Plan& plan, const Sweep& sw, int rq, std::vector<Tmp>& ts,
+                           const std::vector<int>& ts_attach, SweepProgram<R>& P) {
   std::memset(&P.h, 0, sizeof(P.h));
   P.h.n = plan.n;
   P.h.m = sw.m;
@@ -652,7 +654,7 @@ bool finish_program(const Plan& plan, const Sweep& sw, int rq, std::vector<Tmp>&
 // diagonals get a shared-memory phase of their own.  False when the sweep does
 // not fit one program.
 template <typename R>
-bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override) {
+static bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P, int rq_override) {
   const int rq = rq_override > 0 ? rq_override : plan.lane ? kMaxRegQ : reg_qubits_for(sw.m);
   int loc[64];
   for (int q = 0; q < 64; q++) loc[q] = -1;
