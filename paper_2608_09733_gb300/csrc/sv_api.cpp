@@ -655,7 +655,7 @@ namespace sv {
 namespace {
 
 // f(i) for i in 0..n-1 on up to one host thread per core (requests are
-// independent; planning one takes about 0.2 ms).  The error of the lowest
+// independent; planning one takes 0.1 to 0.5 ms).  The error of the lowest
 // index is raised, as a loop would; a thread that cannot be started is done
 // without.
 template <typename F>

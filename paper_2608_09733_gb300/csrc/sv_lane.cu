@@ -26,9 +26,10 @@
 // RY/RZ/CNOT layers 690 -> 162; 14 qubits, 20 layers of U3 and CZ 811 -> 542;
 // complex64, U3 and CNOT ladder of depth 22 on 15 qubits 465 -> 303; 200 one-
 // and 100 two-qubit random matrices on 13 qubits 476 -> 77 (joined matrices,
-// two passes).  A pass of the 12-qubit ansatz waits about 11 cycles an
-// instruction (shared-memory round trips of shuffles and operands), its FP64
-// pipe busy a third of the time: the serial chain still bounds it.
+// two passes).  A pass of the 12-qubit ansatz (36 us, 16 SMs of two warps a
+// scheduler) issues an instruction of each warp every 11 cycles (4.8 of them
+// wait for shared-memory round trips of shuffles and operands, 2.9 for fixed
+// latencies), its FP64 pipe 44 % busy: the serial chain still bounds it.
 #include <cuda_runtime.h>
 
 #include <atomic>
