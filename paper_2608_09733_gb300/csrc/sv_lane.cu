@@ -116,7 +116,9 @@ struct OpWords {
   __device__ __forceinline__ uint32_t k() const { return (a.x >> 8) & 255u; }
   __device__ __forceinline__ uint32_t pos(int i) const { return (a.x >> (16 + 8 * i)) & 255u; }  // i < 2
   __device__ __forceinline__ uint32_t gq(int i) const { return (a.w >> (8 * i)) & 255u; }         // i < 4
-  __device__ __forceinline__ uint32_t rs(int i) const { return (i < 3 ? b.x >> (8 + 8 * i) : b.y) & 255u; }  // i < 4
+  __device__ __forceinline__ uint32_t rs(int i) const {  // i < 5
+    return (i < 3 ? b.x >> (8 + 8 * i) : b.y >> (8 * (i - 3))) & 255u;
+  }
   __device__ __forceinline__ uint32_t lmask() const { return b.z; }
   __device__ __forceinline__ uint32_t lval() const { return b.w; }
   __device__ __forceinline__ uint32_t tmask() const { return c.x; }
@@ -132,6 +134,44 @@ static_assert(offsetof(DevOp, k) == 1 && offsetof(DevOp, pos) == 2 && offsetof(D
                   offsetof(DevOp, xmask) == 40 && offsetof(DevOp, xval) == 48 && offsetof(DevOp, coef) == 56 &&
                   offsetof(DevOp, pad) == 60,
               "OpWords reads DevOp by word");
+
+// A dense matrix of three to five qubits, all on the lane's bits: the 2^k
+// amplitudes of a group sit in one warp.  Row r (the lane's) times the group, by
+// columns r ^ d in Gray-code order of d, so that each step's partner is one
+// shuffle away and the lanes' coefficients M[r][r ^ d] lie in different banks.
+// (Read one by one from the cluster's shared memory, 2^k round trips an
+// amplitude, 100 gates as five-qubit blocks on 16 qubits took 1012 us in
+// complex64, where the one-CTA pass takes 392.)
+template <typename R, int A>
+__device__ __forceinline__ void lane_dense(Cx<R> (&v)[A], const OpWords& op, const Cx<R>* cf, const uint32_t (&tb)[A],
+                                           uint32_t tm, uint32_t tv, bool lane_on, uint32_t lane) {
+  const int k = (int)op.k();
+  uint32_t r = 0, slots = 0;  // slots: five bits a matrix bit
+#pragma unroll
+  for (int i = 0; i < 5; i++) {
+    if (i >= k) continue;
+    r |= ((lane >> op.rs(i)) & 1u) << i;
+    slots |= op.rs(i) << (5 * i);
+  }
+  const Cx<R>* row = cf + (r << k);
+  Cx<R> acc[A];
+  const Cx<R> c0 = row[r];
+#pragma unroll
+  for (int a = 0; a < A; a++) acc[a] = cmul(c0, v[a]);
+  uint32_t d = 0;
+  int mask = 0;
+  for (uint32_t step = 1; step < (1u << k); step++) {
+    const int bit = __ffs((int)step) - 1;
+    d ^= 1u << bit;
+    mask ^= 1 << ((slots >> (5 * bit)) & 31u);
+    const Cx<R> c = row[r ^ d];
+#pragma unroll
+    for (int a = 0; a < A; a++) acc[a] = cfma(c, shfl_partner(v[a], mask), acc[a]);
+  }
+#pragma unroll
+  for (int a = 0; a < A; a++)
+    if (lane_on && (tb[a] & tm) == tv) v[a] = acc[a];
+}
 
 // One register-phase op on the thread's A amplitudes: amplitude a is register
 // combination `lane` of the group whose other local bits are tb[a].
@@ -231,6 +271,8 @@ __device__ __forceinline__ void lane_op(Cx<R> (&v)[A], const OpWords& op, const 
             o = cfma(oth, p, cmul(own, v[a]));
           if (lane_on) v[a] = o;
         }
+      } else if (op.k() >= 3) {
+        lane_dense<R, A>(v, op, cf, tb, tm, tv, lane_on, lane);
       } else {
         const uint32_t r = ((lane >> s0) & 1u) | (((lane >> s1) & 1u) << 1);
         const Cx<R> u0 = cf[r * 4 + r], u1 = cf[r * 4 + (r ^ 1u)], u2 = cf[r * 4 + (r ^ 2u)],
@@ -320,32 +362,16 @@ __device__ __forceinline__ void lane_op(Cx<R> (&v)[A], const OpWords& op, const 
   }
 }
 
-// New value of local amplitude l under a shared-memory op (dense blocks of
-// three to five qubits, wide diagonals), read through ld(l').
-template <typename R, typename Ld>
-__device__ __forceinline__ Cx<R> wide_op(const DevOp& op, const Cx<R>* cf, uint32_t l, uint64_t base, const Ld& ld) {
-  const Cx<R> own = ld(l);
+// Local amplitude l under a shared-memory op: a diagonal of three to five
+// qubits (dense blocks are register ops here).
+template <typename R>
+__device__ __forceinline__ Cx<R> wide_diagonal(const DevOp& op, const Cx<R>* cf, uint32_t l, uint64_t base,
+                                               const Cx<R>& own) {
   if ((l & op.lmask) != op.lval) return own;
-  if (op.kind == OPK_SIGN) return {-own.re, -own.im};
   uint32_t row = 0;  // the op's bits of l (bits outside the tile: fixed)
   for (int i = 0; i < op.k; i++)
     row |= (op.pos[i] != 0xFF ? (l >> op.pos[i]) & 1u : (uint32_t)(base >> op.gq[i]) & 1u) << i;
-  if (op.kind == OPK_DIAG) return cmul(cf[row], own);
-  uint32_t rest = l;
-  for (int i = 0; i < op.k; i++) rest &= ~(1u << op.pos[i]);
-  if (op.kind == OPK_SWAP) {
-    const uint32_t sw = ((row & 1u) << 1) | (row >> 1);
-    return ld(rest | ((sw & 1u) << op.pos[0]) | ((sw >> 1) << op.pos[1]));
-  }
-  if (op.kind == OPK_ANTIDIAG) return cmul(cf[row], ld(l ^ (1u << op.pos[0])));
-  const uint32_t dim = 1u << op.k;
-  Cx<R> acc = {R(0), R(0)};
-  for (uint32_t c = 0; c < dim; c++) {
-    uint32_t at = rest;
-    for (int i = 0; i < op.k; i++) at |= ((c >> i) & 1u) << op.pos[i];
-    acc = cfma(cf[row * dim + c], ld(at), acc);
-  }
-  return acc;
+  return cmul(cf[row], own);
 }
 
 // One pass: cluster t of 2^log_c CTAs takes tile t.  A warp holds A groups of
@@ -417,9 +443,8 @@ __global__ void __launch_bounds__(32 * kLaneWarps)
       for (int a = 0; a < A; a++) {
         const uint32_t l = (first_group + a) * 32u + lane;
         at[a] = addr_of(l);
-        v[a] = wide_op<R>(op, cf, l, base, [&](uint32_t x) { return ld_peer(addr_of(x), R(0)); });
+        v[a] = wide_diagonal<R>(op, cf, l, base, ld_peer(at[a], R(0)));
       }
-      tile_sync(log_c);  // every amplitude has been read
     }
 #pragma unroll
     for (int a = 0; a < A; a++) st_peer(at[a], v[a]);

@@ -740,15 +740,15 @@ bool lane_sizes(int n, const sv_exec_opts& opts) {
 }
 
 // Complex64 states of two and four cluster tiles (15 and 16 qubits): a short
-// circuit of one-qubit gates and diagonals takes the general pass, whose one or
-// two wider passes run few phases.  U3 and CZ on 16 qubits, us, cluster against
+// circuit of one-qubit gates and narrow diagonals takes the general pass, whose
+// one or two wider passes run few phases.  U3 and CZ on 16 qubits, us, cluster against
 // general: 2 layers (62 gates) 36.9 and 28.6, 5 layers (155) 66.5 and 51.7, 6
 // layers (186) 65.9 and 64.1, then within a tenth (20 layers 208 and 200); with
 // flips (RY RZ CNOT, 1 layer) 28.0 and 31.6, with two-qubit matrices 20.8 and
 // 35.3.  The line is at 200 operations.
 static bool short_without_flips(const std::vector<LOp>& ops) {
   return ops.size() < 200 && std::all_of(ops.begin(), ops.end(), [](const LOp& op) {
-           return op.kind == OPK_DIAG || ((op.kind == OPK_DENSE || op.kind == OPK_REAL) && op.k == 1);
+           return op.kind == OPK_DIAG ? op.k <= 2 : (op.kind == OPK_DENSE || op.kind == OPK_REAL) && op.k == 1;
          });
 }
 

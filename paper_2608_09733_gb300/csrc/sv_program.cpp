@@ -787,7 +787,8 @@ static bool build_program(const Plan& plan, const Sweep& sw, SweepProgram<R>& P,
     }
     if (op.kind == OPK_ANTIDIAG && op.m.size() == 2 && op.m[0] == cplx(1.0) && op.m[1] == cplx(1.0)) d.pad = 1;
     const bool wide = (op.kind == OPK_DENSE || op.kind == OPK_REAL) ? op.k >= 3 : (diag && d.kind == OPK_DIAG && op.k >= 3);
-    t.smem = !reg_ok || wide;
+    // dense blocks are register ops of the cluster pass (its lanes hold five qubits)
+    t.smem = !reg_ok || (wide && !(plan.lane && !diag));
   }
 
   // The order of the ops over the phases.  A phase takes, in order, every op
@@ -1007,6 +1008,19 @@ void emulate_reg_op(const SweepProgram<R>& P, const DevOp& op, uint32_t code, in
           a = cz(cf[0]) * a0 + cz(cf[1]) * b0;
           b = cz(cf[2]) * a0 + cz(cf[3]) * b0;
         });
+      } else if (op.k >= 3) {
+        const int dim = 1 << op.k;
+        auto at = [&](int j, int r) {  // combination j with the matrix bits of r
+          for (int i = 0; i < op.k; i++) j = (j & ~(1 << op.rs[i])) | (((r >> i) & 1) << op.rs[i]);
+          return j;
+        };
+        for (int j = 0; j < NR; j++) {
+          if (at(j, 0) != j || ((uint32_t)j & rm) != rv) continue;
+          std::vector<zc> y(dim, 0.0);
+          for (int r = 0; r < dim; r++)
+            for (int c = 0; c < dim; c++) y[r] += cz(cf[r * dim + c]) * v[at(j, c)];
+          for (int r = 0; r < dim; r++) v[at(j, r)] = y[r];
+        }
       } else {
         const int A = op.rs[0], B = op.rs[1];
         for (int j = 0; j < NR; j++) {
