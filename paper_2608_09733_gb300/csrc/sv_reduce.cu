@@ -426,12 +426,17 @@ size_t expect_terms_scratch_doubles(int n, int n_terms) {
 }
 
 // Blocks of a state's read-out: a warp a chunk; blocks of one warp until the
-// grid holds four blocks an SM over the whole batch (a small state spreads over
-// the SMs), then of up to eight.
+// grid holds a block an SM over the whole batch (a small state spreads over the
+// SMs), then of up to eight.  More than 4096 chunks take up to four blocks an
+// SM: the finish adds a row a block, which is most of the time of a small state
+// (complex64, us, four blocks an SM against one: 18 qubits 12.5 and 12.5, 20
+// qubits 19.7 and 14.5, 23 qubits 24.8 and 18.7, 24 qubits 41 and 46, 26 qubits
+// 95 and 137).
 static int z_all_blocks(int n, int chunk_bits, int batch, int* warps) {
   if (n < chunk_bits) return 1;
   const uint64_t chunks = 1ull << (n - chunk_bits);
-  const uint64_t most = ((uint64_t)red_grid() + batch - 1) / batch;
+  const uint64_t blocks = chunks * batch <= 4096 ? device_sm_count() : red_grid();
+  const uint64_t most = (blocks + batch - 1) / batch;
   const uint64_t g = chunks < most ? chunks : most;
   *warps = 1;
   while (*warps < kRedWarps && chunks > g * *warps) *warps *= 2;
