@@ -256,24 +256,7 @@ __device__ __forceinline__ void lane_op(Cx<R> (&v)[A], const OpWords& op, const 
       break;
     case OPK_DENSE:
     case OPK_REAL:
-      if (op.k() == 1) {
-        const bool up = (lane >> s0) & 1u;
-        const Cx<R> own = cf[up ? 3 : 0], oth = cf[up ? 2 : 1];
-        const bool real = kind == OPK_REAL;
-#pragma unroll
-        for (int a = 0; a < A; a++) {
-          if ((tb[a] & tm) != tv) continue;  // the same for the warp
-          const Cx<R> p = shfl_partner(v[a], 1 << s0);
-          Cx<R> o;
-          if (real)
-            o = {fma(own.re, v[a].re, oth.re * p.re), fma(own.re, v[a].im, oth.re * p.im)};
-          else
-            o = cfma(oth, p, cmul(own, v[a]));
-          if (lane_on) v[a] = o;
-        }
-      } else if (op.k() >= 3) {
-        lane_dense<R, A>(v, op, cf, tb, tm, tv, lane_on, lane);
-      } else {
+      if (op.k() == 2) {
         const uint32_t r = ((lane >> s0) & 1u) | (((lane >> s1) & 1u) << 1);
         const Cx<R> u0 = cf[r * 4 + r], u1 = cf[r * 4 + (r ^ 1u)], u2 = cf[r * 4 + (r ^ 2u)],
                     u3 = cf[r * 4 + (r ^ 3u)];
@@ -288,6 +271,23 @@ __device__ __forceinline__ void lane_op(Cx<R> (&v)[A], const OpWords& op, const 
           o = cfma(u3, p3, o);
           if (lane_on) v[a] = o;
         }
+      } else if (op.k() == 1) {
+        const bool up = (lane >> s0) & 1u;
+        const Cx<R> own = cf[up ? 3 : 0], oth = cf[up ? 2 : 1];
+        const bool real = kind == OPK_REAL;
+#pragma unroll
+        for (int a = 0; a < A; a++) {
+          if ((tb[a] & tm) != tv) continue;  // the same for the warp
+          const Cx<R> p = shfl_partner(v[a], 1 << s0);
+          Cx<R> o;
+          if (real)
+            o = {fma(own.re, v[a].re, oth.re * p.re), fma(own.re, v[a].im, oth.re * p.im)};
+          else
+            o = cfma(oth, p, cmul(own, v[a]));
+          if (lane_on) v[a] = o;
+        }
+      } else {
+        lane_dense<R, A>(v, op, cf, tb, tm, tv, lane_on, lane);
       }
       break;
     case OPK_ANTIDIAG: {
